@@ -12,11 +12,11 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 
-// Dynamic shared memory of a CTA (no device work): the coarsest level's dense
-// matrix; then the arrays that the cycles read on the small coarse levels
+// Dynamic shared memory of a CTA (no device work): the coarsest level's
+// factored matrix; then the arrays that the cycles read on the small coarse levels
 // that warp 0 runs alone (levels l >= 1 with at most WARP_CELLS cells: the
 // multigrid arrays, and for FP64 the coarsest level's faces and diagonal,
-// which the direct solve assembles); then the corrections dp of as many of the other levels
+// from which the matrix is assembled); then the corrections dp of as many of the other levels
 // (coarsest first) as fit the budget of the launch shape (one 1024-thread CTA
 // per SM may use ~220 KB, two 512-thread CTAs ~104 KB each, four 256-thread
 // CTAs ~50 KB each, eight 128-thread CTAs ~24 KB each), so that the
@@ -65,6 +65,10 @@ static void plan_smem(FParams& P, int nt) {
         P.osm[l] = (long long)off;
         off += bytes;
     }
+    // the finest FP64 level's second red half goes with its dp
+    P.osm_alt = -1;
+    const size_t half = al16((size_t)P.nx[0] * P.nz[0] / 2 * w);
+    if (!P.mixed && P.osm[0] >= 0 && off + half <= budget) { P.osm_alt = (long long)off; off += half; }
     P.smem_bytes = (long long)off;
 }
 
@@ -87,9 +91,10 @@ static int fused_setup(const rich_problem_t* pb, int S, FParams& P, int ckpt_eve
             P.o64[l][k] = (long long)off; off = al256(off + bytes);
         }
         for (int k = 0; k < NMG; ++k) {
-            // FP64: wE wW wN wS q f dp D ; FP32: Tx Tz - D q f dp - (slots B_2, B_7 unused)
-            if (mixed && (k == B_2 || k == B_7)) { P.omg[l][k] = -1; continue; }
-            P.omg[l][k] = (long long)off; off = al256(off + nc * w);
+            // FP64: wE wW wN wS q f dp D alt (the half array alt on the finest level
+            // only); FP32: Tx Tz - D q f dp - -
+            if (mixed ? (k == B_2 || k == B_7 || k == B_ALT) : (l > 0 && k == B_ALT)) { P.omg[l][k] = -1; continue; }
+            P.omg[l][k] = (long long)off; off = al256(off + (k == B_ALT ? (nc + 1) / 2 : nc) * w);
         }
         lx /= 2; lz /= 2;
     }

@@ -52,8 +52,9 @@ constexpr int ADJ_M = 12;                // GMRES restart length of the adjoint'
 // FP64 unscaled operator (all levels): faces, mass term, diagonal, Dirichlet faces
 enum { A_TX, A_TZ, A_CDT, A_D, A_TBT, A_TBB, N64 };
 // multigrid arrays in the cycle precision, colour-split on every level but
-// the coarsest.  FP64: wE wW wN wS q=1/D fh dp D.  FP32: Tx Tz - D 1/D f dp -.
-enum { B_0, B_1, B_2, B_3, B_4, B_5, B_6, B_7, NMG };
+// the coarsest.  FP64: wE wW wN wS q=1/D fh dp D alt (the second red half alt
+// of dp on the finest level only).  FP32: Tx Tz - D 1/D f dp - -.
+enum { B_0, B_1, B_2, B_3, B_4, B_5, B_6, B_7, B_ALT, NMG };
 
 struct FParams {
     int S, nlev, mixed;
@@ -63,6 +64,7 @@ struct FParams {
     long long omg[MAXL][NMG];
     long long osm[MAXL];                    // level's dp in dynamic shared memory at this
                                             // byte offset (-1: in the slot)
+    long long osm_alt;                      // likewise the finest level's second red half
     int lw;                                 // first level run by warp 0 alone (nlev: none)
     long long s64[MAXL][N64];               // levels >= lw: every array in dynamic shared
     long long smg[MAXL][NMG];               // memory at these byte offsets (-1: not there)
@@ -106,7 +108,7 @@ struct FParams {
 // allow a kernel `bytes` of dynamic shared memory above the 48 KB default; the
 // attribute is set once per (kernel, device, larger size)
 inline int allow_dyn_smem(const void* kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return 0;
+    if (bytes <= 32 * 1024) return 0;        // with the kernel's static arrays within the 48 KB default
     struct Grant { const void* k; int dev; size_t bytes; };
     static Grant grants[128];
     static int ngrants = 0;
@@ -196,15 +198,11 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
     v = warp_max_u64(v);
     if (lane == 0) red[wid] = v;
     __syncthreads();
-    if (wid == 0) {
-        v = lane < nw ? red[lane] : 0ull;
-        v = warp_max_u64(v);
-        if (lane == 0) red[32] = v;
-    }
+    // every warp reduces the partials itself: one barrier less than a
+    // broadcast of warp 0's result
+    v = warp_max_u64(lane < nw ? red[lane] : 0ull);
     __syncthreads();
-    unsigned long long r = red[32];
-    __syncthreads();
-    return r;
+    return v;
 }
 
 struct Lv64 {
@@ -214,7 +212,8 @@ struct Lv64 {
 };
 
 // multigrid level in cycle precision T.  FP64 (scaled): c = {wE, wW, wN, wS},
-// q = 1/D, f = f/D (the coarsest level keeps f unscaled for the direct solve).
+// q = 1/D (below the finest level 1/(4 D), see restrict_cells), f = f/D (the
+// coarsest level keeps f unscaled for the direct solve).
 // FP32 (unscaled): c = {Tx, Tz, -, -}, q = 1/D, f = f.
 // Layout: every level that is smoothed stores its cells colour-split, the red
 // cells ((i + j) even) first and then the black ones, each half row-major with
@@ -222,12 +221,16 @@ struct Lv64 {
 // (H = hx nz).  A half-sweep then reads its own cells, and the neighbours of
 // the other colour, at unit stride (no shared-memory bank conflicts, full
 // sectors from L2).  The coarsest level (direct solve; its sides may be odd)
-// keeps the natural row-major order (H = 0).
+// keeps the natural row-major order (H = 0).  The two halves of dp have a
+// pointer each, both to be indexed like the other arrays: dp (red cells; all of
+// them on the coarsest level) and db (black cells: H before their first one).
+// They point at one array, except on the finest FP64 level, whose second red
+// half, alt, swaps with dp.
 template <typename T>
 struct Lv {
     int nx, nz, hx, nc, H;
     unsigned mnx, mhx;
-    T *c0, *c1, *c2, *c3, *D, *q, *f, *dp;
+    T *c0, *c1, *c2, *c3, *D, *q, *f, *dp, *db, *alt;
 };
 
 // storage index of cell (i, j) on a level
@@ -236,17 +239,19 @@ __device__ __forceinline__ int sidx(const Lv<T>& L, int i, int j) {
     return L.H ? ((i + j) & 1) * L.H + j * L.hx + (i >> 1) : j * L.nx + i;
 }
 
-// storage indices of cell (i, j) and of its east, west, north and south
-// neighbours (valid where the neighbour exists)
-struct Nb { int own, e, w, n, s; };
+// the correction at cell (i, j)
 template <typename T>
-__device__ __forceinline__ Nb nb_of(const Lv<T>& L, int i, int j) {
-    if (L.H) {
-        const int col = (i + j) & 1, c = j * L.hx + (i >> 1), oth = (1 - col) * L.H + c;
-        return Nb{col * L.H + c, oth + (i & 1), oth - 1 + (i & 1), oth + L.hx, oth - L.hx};
-    }
-    const int P = j * L.nx + i;
-    return Nb{P, P + 1, P - 1, P + L.nx, P - L.nx};
+__device__ __forceinline__ T dp_at(const Lv<T>& L, int i, int j) {
+    return (((i + j) & 1) && L.H ? L.db : L.dp)[sidx(L, i, j)];
+}
+
+// storage indices of a cell of a colour-split level (col 0 red, 1 black; c its
+// place in its colour's half, i its column) and of its east, west, north and
+// south neighbours (valid where the neighbour exists)
+struct Nb { int own, e, w, n, s; };
+__device__ __forceinline__ Nb nb_half(int col, int c, int i, int hx, int H) {
+    const int oth = (1 - col) * H + c;
+    return Nb{col * H + c, oth + (i & 1), oth - 1 + (i & 1), oth + hx, oth - hx};
 }
 
 template <typename T> struct Scaled { static constexpr bool value = sizeof(T) == 8; };
@@ -268,10 +273,10 @@ struct GWarp {
 };
 
 // Gauss-Seidel value of a cell (storage indices b) from its current
-// neighbours, with the level's arrays passed as restrict-qualified pointers:
-// every caller reads dp only at cells that it does not write in the same pass
-// (see rbgs_cells), so the compiler may keep several cells' loads in flight
-// ahead of the stores.
+// neighbours, in the half `o` of dp, with the level's arrays passed as
+// restrict-qualified pointers: every caller reads dp only at cells that it does
+// not write in the same pass (see rbgs_cells), so the compiler may keep several
+// cells' loads in flight ahead of the stores.
 //   FP64 (scaled): c0..c3 = wE, wW, wN, wS; value f + sum w dp_nb.
 //   FP32 (unscaled): c0 = Tx (east face), c1 = Tz (north face); the west and
 //   south faces are the neighbours'; value (f + sum T dp_nb) / D.
@@ -279,78 +284,166 @@ template <typename T>
 __device__ __forceinline__ T gs_at(const Nb& b, bool hE, bool hW, bool hN, bool hS, const T* __restrict__ f,
                                    const T* __restrict__ c0, const T* __restrict__ c1,
                                    const T* __restrict__ c2, const T* __restrict__ c3,
-                                   const T* __restrict__ q, const T* __restrict__ dp) {
+                                   const T* __restrict__ q, const T* __restrict__ o) {
     if constexpr (Scaled<T>::value) {
         T v = f[b.own];
-        if (hE) v += c0[b.own] * dp[b.e];
-        if (hW) v += c1[b.own] * dp[b.w];
-        if (hN) v += c2[b.own] * dp[b.n];
-        if (hS) v += c3[b.own] * dp[b.s];
+        if (hE) v += c0[b.own] * o[b.e];
+        if (hW) v += c1[b.own] * o[b.w];
+        if (hN) v += c2[b.own] * o[b.n];
+        if (hS) v += c3[b.own] * o[b.s];
         return v;
     } else {
         T t = T(0);
-        if (hE) t += c0[b.own] * dp[b.e];
-        if (hW) t += c0[b.w] * dp[b.w];
-        if (hN) t += c1[b.own] * dp[b.n];
-        if (hS) t += c1[b.s] * dp[b.s];
+        if (hE) t += c0[b.own] * o[b.e];
+        if (hW) t += c0[b.w] * o[b.w];
+        if (hN) t += c1[b.own] * o[b.n];
+        if (hS) t += c1[b.s] * o[b.s];
         return (f[b.own] + t) * q[b.own];
     }
 }
 
-// residual f - A dp at a cell (unscaled): FP64 D (value - dp), FP32
-// f - (D dp - sum T dp_nb)
+// residual f - A dp (unscaled) of a cell whose correction is d: FP64
+// D (value - d), FP32 f - (D d - sum T dp_nb)
 template <typename T>
 __device__ __forceinline__ T resid_at(const Nb& b, bool hE, bool hW, bool hN, bool hS,
                                       const T* __restrict__ f, const T* __restrict__ c0,
                                       const T* __restrict__ c1, const T* __restrict__ c2,
                                       const T* __restrict__ c3, const T* __restrict__ q,
-                                      const T* __restrict__ D, const T* __restrict__ dp) {
+                                      const T* __restrict__ D, const T* __restrict__ o, T d) {
     if constexpr (Scaled<T>::value) {
-        return D[b.own] * (gs_at<T>(b, hE, hW, hN, hS, f, c0, c1, c2, c3, q, dp) - dp[b.own]);
+        return D[b.own] * (gs_at<T>(b, hE, hW, hN, hS, f, c0, c1, c2, c3, q, o) - d);
     } else {
         T t = T(0);
-        if (hE) t += c0[b.own] * dp[b.e];
-        if (hW) t += c0[b.w] * dp[b.w];
-        if (hN) t += c1[b.own] * dp[b.n];
-        if (hS) t += c1[b.s] * dp[b.s];
-        return f[b.own] - (D[b.own] * dp[b.own] - t);
+        if (hE) t += c0[b.own] * o[b.e];
+        if (hW) t += c0[b.w] * o[b.w];
+        if (hN) t += c1[b.own] * o[b.n];
+        if (hS) t += c1[b.s] * o[b.s];
+        return f[b.own] - (D[b.own] * d - t);
     }
 }
 
+// a + b, not contracted with the product that gave a or b: the one-cell and the
+// two-cell loops of a level give the same bits
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+
+// 16-byte accesses: two FP64 or four FP32 neighbours of one colour
+__device__ __forceinline__ void ld_vec(const double* p, double (&v)[2]) {
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void ld_vec(const float* p, float (&v)[4]) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void st_vec(double* p, const double (&v)[2]) {
+    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+}
+__device__ __forceinline__ void st_vec(float* p, const float (&v)[4]) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <typename T> struct Vec { static constexpr int W = 16 / sizeof(T); };
+
+// Gauss-Seidel values of W = 2 (FP64) or 4 (FP32) cells c, c + 1, ... of one
+// colour in row j (c a multiple of W, hx too: 16-byte aligned), bit for bit
+// those of gs_at.  The half-sweeps are bound by the latency of their loads and
+// by the FP64 pipe (a warp's DFMA holds its quarter of the SM for 64 cycles),
+// so a thread's loads are 16 bytes wide and all issued before the arithmetic:
+// 9 (FP64) or 11 (FP32) loads instead of 18 or 40.  A 128^2 batch of 608
+// samples, two steps, 512 threads: FP32 cycles 399 -> 310 ms, FP64 650 -> 590 ms
+// (with the first red half-sweep taken from the norm and the black-only
+// prolongation).  Missing neighbours count as zero; their face coefficient is
+// zero too.
 template <typename T>
-__device__ __forceinline__ T resid_cell(const Lv<T>& L, int i, int j) {
-    return resid_at<T>(nb_of(L, i, j), i < L.nx - 1, i > 0, j < L.nz - 1, j > 0, L.f, L.c0, L.c1, L.c2, L.c3,
-                       L.q, L.D, L.dp);
+__device__ __forceinline__ void gs_vec(int c, int j, int nz, int hx, int H, int colour, const T* __restrict__ f,
+                                       const T* __restrict__ c0, const T* __restrict__ c1,
+                                       const T* __restrict__ c2, const T* __restrict__ c3,
+                                       const T* __restrict__ q, const T* __restrict__ o, T (&v)[Vec<T>::W]) {
+    constexpr int W = Vec<T>::W;
+    const int k = c - j * hx, s = (j + colour) & 1, own = colour * H + c, oth = (1 - colour) * H + c;
+    const bool hN = j < nz - 1, hS = j > 0, hX = s ? k + W < hx : k > 0;
+    const int x = s ? oth + W : oth - 1;              // the neighbour beside the W in the own row
+    T a0[W], a1[W], a2[W], a3[W], qq[W], m[W], n[W] = {}, u[W] = {}, side = T(0), wside = T(0), cw[W], cs[W] = {};
+    ld_vec(f + own, v);
+    ld_vec(c0 + own, a0);
+    ld_vec(c1 + own, a1);
+    if constexpr (Scaled<T>::value) {
+        ld_vec(c2 + own, a2);
+        ld_vec(c3 + own, a3);
+    } else {
+        ld_vec(q + own, qq);
+        ld_vec(c0 + oth, cw);
+        if (hS) ld_vec(c1 + oth - hx, cs);
+        if (!s && hX) wside = c0[x];
+    }
+    ld_vec(o + oth, m);
+    if (hN) ld_vec(o + oth + hx, n);
+    if (hS) ld_vec(o + oth - hx, u);
+    if (hX) side = o[x];
+#pragma unroll
+    for (int t = 0; t < W; ++t) {
+        const T e = !s ? m[t] : t + 1 < W ? m[t + 1 < W ? t + 1 : 0] : side;
+        const T w = s ? m[t] : t > 0 ? m[t > 0 ? t - 1 : 0] : side;
+        if constexpr (Scaled<T>::value) {
+            v[t] = fma(a0[t], e, v[t]);
+            v[t] = fma(a1[t], w, v[t]);
+            v[t] = fma(a2[t], n[t], v[t]);
+            v[t] = fma(a3[t], u[t], v[t]);
+        } else {
+            const T tw = s ? cw[t] : t > 0 ? cw[t > 0 ? t - 1 : 0] : wside;
+            T z = T(0);
+            z += a0[t] * e;
+            z += tw * w;
+            z += a1[t] * n[t];
+            z += cs[t] * u[t];
+            v[t] = (v[t] + z) * qq[t];
+        }
+    }
+}
+
+// whether a level's loops take W cells of a colour at a time: aligned rows, and
+// still a cell for every thread of the group (a level with fewer cells is
+// faster spread over more warps, one cell a thread)
+template <typename T, typename G>
+__device__ __forceinline__ bool wide(int hx, int H) {
+    return hx % Vec<T>::W == 0 && H >= Vec<T>::W * G::size();
 }
 
 // one colour of red-black Gauss-Seidel over a colour-split level (red:
 // i + j even).  The corrections are read through one restrict-qualified view
-// and written through another: a half-sweep writes cells of one colour and
-// reads only cells of the other, so the two views never touch one element.
+// (the other colour's half) and written through another (its own).
 template <typename T, typename G>
 __device__ __forceinline__ void rbgs_cells(int nx, int nz, int hx, int H, unsigned mhx, int colour,
                                            const T* __restrict__ f, const T* __restrict__ c0,
                                            const T* __restrict__ c1, const T* __restrict__ c2,
                                            const T* __restrict__ c3, const T* __restrict__ q,
-                                           const T* __restrict__ dpr, T* __restrict__ dpw) {
-#pragma unroll 4
-    for (int c = G::rank(); c < H; c += G::size()) {
-        const int j = fdiv(c, hx, mhx);
-        const int i = 2 * (c - j * hx) + ((j + colour) & 1);
-        const int oth = (1 - colour) * H + c;
-        const Nb b{colour * H + c, oth + (i & 1), oth - 1 + (i & 1), oth + hx, oth - hx};
-        dpw[b.own] = gs_at<T>(b, i < nx - 1, i > 0, j < nz - 1, j > 0, f, c0, c1, c2, c3, q, dpr);
+                                           const T* __restrict__ o, T* __restrict__ own) {
+    if (wide<T, G>(hx, H)) {
+        for (int c = Vec<T>::W * G::rank(); c < H; c += Vec<T>::W * G::size()) {
+            T v[Vec<T>::W];
+            gs_vec<T>(c, fdiv(c, hx, mhx), nz, hx, H, colour, f, c0, c1, c2, c3, q, o, v);
+            st_vec(own + colour * H + c, v);
+        }
+    } else {
+#pragma unroll 1
+        for (int c = G::rank(); c < H; c += G::size()) {
+            const int j = fdiv(c, hx, mhx);
+            const int i = 2 * (c - j * hx) + ((j + colour) & 1);
+            const Nb b = nb_half(colour, c, i, hx, H);
+            own[b.own] = gs_at<T>(b, i < nx - 1, i > 0, j < nz - 1, j > 0, f, c0, c1, c2, c3, q, o);
+        }
     }
     G::sync();
 }
 
 template <typename T, typename G>
 __device__ __forceinline__ void rbgs(const Lv<T>& L, int colour) {
-    rbgs_cells<T, G>(L.nx, L.nz, L.hx, L.H, L.mhx, colour, L.f, L.c0, L.c1, L.c2, L.c3, L.q, L.dp, L.dp);
+    rbgs_cells<T, G>(L.nx, L.nz, L.hx, L.H, L.mhx, colour, L.f, L.c0, L.c1, L.c2, L.c3, L.q,
+                     colour ? L.dp : L.db, colour ? L.db : L.dp);
 }
 
 template <typename T, typename G>
-__device__ __forceinline__ void prolong(const Lv<T>& F, const Lv<T>& C);
+__device__ __forceinline__ void prolong(const Lv<T>& F, const Lv<T>& C, bool black_only);
 
 // nu red-black sweeps; with seeded true the first red half-sweep is skipped
 // because the restriction already stored its result (see restrict_cells)
@@ -365,7 +458,7 @@ __device__ __forceinline__ void smooth(const Lv<T>& L, int nu, bool seeded = fal
 // prolongation and post-smoothing of level l from level l+1
 template <typename T, typename G>
 __device__ __forceinline__ void prolong_smooth(const Lv<T>& F, const Lv<T>& C, int nu2) {
-    prolong<T, G>(F, C);
+    prolong<T, G>(F, C, nu2 > 0);
     smooth<T, G>(F, nu2);
 }
 
@@ -374,47 +467,90 @@ __device__ __forceinline__ void prolong_smooth(const Lv<T>& F, const Lv<T>& C, i
 // fine level, writes the coarse one (distinct arrays: restrict views).  The
 // fine level is colour-split: the children of coarse cell (I, J) are the red
 // cells r0 = 2J hx + I and r0 + hx and the black cells H + r0, H + r0 + hx.
+// FP64: the coarse level's cq is 1/(4 D), so that one multiplication takes the
+// mean and scales the right-hand side.
 // The coarse correction starts at zero; when the coarse level is smoothed
 // next (seed), its red cells get at once the value the first red half-sweep
 // would compute from all-zero neighbours, f q (FP64: the scaled f), so that
-// half-sweep is skipped.
+// half-sweep is skipped; its black cells are overwritten before they are read.
 template <typename T, typename G>
-__device__ __forceinline__ void restrict_cells(const Lv<T>& F, const Lv<T>& C, bool red_only, bool scale, bool seed,
+__device__ __forceinline__ void restrict_cells(const Lv<T>& F, const Lv<T>& C, bool red_only, bool coarsest, bool seed,
                                                const T* __restrict__ f, const T* __restrict__ c0,
                                                const T* __restrict__ c1, const T* __restrict__ c2,
                                                const T* __restrict__ c3, const T* __restrict__ q,
-                                               const T* __restrict__ D, const T* __restrict__ dp,
-                                               const T* __restrict__ cq, T* __restrict__ cf, T* __restrict__ cdp) {
+                                               const T* __restrict__ D, const T* __restrict__ dr,
+                                               const T* __restrict__ db, const T* __restrict__ cq,
+                                               T* __restrict__ cf, T* __restrict__ cdp) {
     const int nx = F.nx, nz = F.nz, hx = F.hx, H = F.H;
+    if constexpr (Scaled<T>::value) {
+        // two coarse cells a thread, 16-byte loads (see gs_vec); the black rows
+        // j and j + 1 serve both red rows
+        if (red_only && !coarsest && wide<T, G>(hx, C.nc)) {
+            for (int c = 2 * G::rank(); c < C.nc; c += 2 * G::size()) {
+                const int J = fdiv(c, C.nx, C.mnx), I = c - J * C.nx, j = 2 * J, r0 = j * hx + I, r1 = r0 + hx;
+                double bs[2] = {}, b0[2], b1[2], bn[2] = {}, lo = 0.0, hi = 0.0, v0[2], v1[2], a[2], d[2];
+                ld_vec(db + H + r0, b0);
+                ld_vec(db + H + r1, b1);
+                if (j > 0) ld_vec(db + H + r0 - hx, bs);
+                if (j + 2 < nz) ld_vec(db + H + r1 + hx, bn);
+                if (I > 0) lo = db[H + r0 - 1];
+                if (I + 2 < hx) hi = db[H + r1 + 2];
+                ld_vec(f + r0, v0);
+                ld_vec(f + r1, v1);
+                const double e0[2] = {b0[0], b0[1]}, w0[2] = {lo, b0[0]}, e1[2] = {b1[1], hi}, w1[2] = {b1[0], b1[1]};
+                auto face = [&](const double* w, const double (&x0)[2], const double (&x1)[2]) {
+                    ld_vec(w + r0, a);
+                    v0[0] = fma(a[0], x0[0], v0[0]); v0[1] = fma(a[1], x0[1], v0[1]);
+                    ld_vec(w + r1, a);
+                    v1[0] = fma(a[0], x1[0], v1[0]); v1[1] = fma(a[1], x1[1], v1[1]);
+                };
+                face(c0, e0, e1);
+                face(c1, w0, w1);
+                face(c2, b1, bn);
+                face(c3, bs, b0);
+                ld_vec(dr + r0, d); v0[0] -= d[0]; v0[1] -= d[1];
+                ld_vec(dr + r1, d); v1[0] -= d[0]; v1[1] -= d[1];
+                ld_vec(D + r1, d); v1[0] *= d[0]; v1[1] *= d[1];
+                ld_vec(D + r0, d);
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int cs = sidx(C, I + t, J);
+                    const double fc = cq[cs] * add_rn(__dmul_rn(d[t], v0[t]), v1[t]);
+                    cf[cs] = fc;
+                    if (!seed) cdp[cs] = 0.0;
+                    else if (!((I + t + J) & 1)) cdp[cs] = fc;
+                }
+            }
+            G::sync();
+            return;
+        }
+    }
 #pragma unroll(Scaled<T>::value ? 1 : 2)
     for (int c = G::rank(); c < C.nc; c += G::size()) {
         const int J = fdiv(c, C.nx, C.mnx), I = c - J * C.nx;
-        const int i = 2 * I, j = 2 * J, r0 = j * hx + I;
+        const int i = 2 * I, j = 2 * J, r0 = j * hx + I, r1 = r0 + hx;
         // red (i, j): neighbours black; red (i+1, j+1) likewise
-        const Nb b00{r0, H + r0, H + r0 - 1, H + r0 + hx, H + r0 - hx};
-        const Nb b11{r0 + hx, H + r0 + hx + 1, H + r0 + hx, H + r0 + 2 * hx, H + r0};
-        const T r00 = resid_at<T>(b00, true, i > 0, true, j > 0, f, c0, c1, c2, c3, q, D, dp);
-        const T r11 = resid_at<T>(b11, i + 1 < nx - 1, true, j + 1 < nz - 1, true, f, c0, c1, c2, c3, q, D, dp);
+        const T r11 = resid_at<T>(nb_half(0, r1, i + 1, hx, H), i + 1 < nx - 1, true, j + 1 < nz - 1, true, f, c0,
+                                  c1, c2, c3, q, D, db, dr[r1]);
+        const T r00 = resid_at<T>(nb_half(0, r0, i, hx, H), true, i > 0, true, j > 0, f, c0, c1, c2, c3, q, D, db,
+                                  dr[r0]);
         T sum;
         if (red_only) {
-            sum = r00 + r11;
+            sum = add_rn(r00, r11);
         } else {
-            const Nb b10{H + r0, r0 + 1, r0, r0 + hx, r0 - hx};
-            const Nb b01{H + r0 + hx, r0 + hx, r0 + hx - 1, r0 + 2 * hx, r0};
-            const T r10 = resid_at<T>(b10, i + 1 < nx - 1, true, true, j > 0, f, c0, c1, c2, c3, q, D, dp);
-            const T r01 = resid_at<T>(b01, true, i > 0, j + 1 < nz - 1, true, f, c0, c1, c2, c3, q, D, dp);
+            const T r10 = resid_at<T>(nb_half(1, r0, i + 1, hx, H), i + 1 < nx - 1, true, true, j > 0, f, c0, c1, c2,
+                                      c3, q, D, dr, db[H + r0]);
+            const T r01 = resid_at<T>(nb_half(1, r1, i, hx, H), true, i > 0, j + 1 < nz - 1, true, f, c0, c1, c2, c3,
+                                      q, D, dr, db[H + r1]);
             sum = r00 + r10 + r01 + r11;
         }
         const int cs = sidx(C, I, J);
-        T fc = T(0.25) * sum;
-        if (scale) fc *= cq[cs];
+        const T fc = Scaled<T>::value && !coarsest ? sum * cq[cs] : T(0.25) * sum;
         cf[cs] = fc;
-        T d0 = T(0);
-        if (seed && !((I + J) & 1)) {
-            if constexpr (Scaled<T>::value) d0 = fc;
-            else d0 = fc * cq[cs];
+        if (!coarsest) {                              // (the coarsest solve writes its own)
+            if (!seed) cdp[cs] = T(0);
+            else if (!((I + J) & 1)) cdp[cs] = Scaled<T>::value ? fc : fc * cq[cs];
         }
-        cdp[cs] = d0;
     }
     G::sync();
 }
@@ -422,33 +558,58 @@ __device__ __forceinline__ void restrict_cells(const Lv<T>& F, const Lv<T>& C, b
 template <typename T, typename G>
 __device__ __forceinline__ void resid_restrict(const Lv<T>& F, const Lv<T>& C, bool red_only, bool coarsest,
                                                bool seed = false) {
-    restrict_cells<T, G>(F, C, red_only, Scaled<T>::value && !coarsest, seed && !coarsest, F.f, F.c0, F.c1, F.c2,
-                         F.c3, F.q, F.D, F.dp, C.q, C.f, C.dp);
+    restrict_cells<T, G>(F, C, red_only, coarsest, seed, F.f, F.c0, F.c1, F.c2, F.c3, F.q, F.D, F.dp, F.db,
+                         C.q, C.f, C.dp);
 }
 
 // piecewise-constant prolongation and correction: each coarse cell adds its
-// value to its own four children, so no two iterations touch one element
+// value to its own four children, so no two iterations touch one element.  When
+// a red half-sweep follows (black_only) the red children are left alone: that
+// half-sweep replaces them without reading them.
 template <typename T, typename G>
-__device__ __forceinline__ void prolong(const Lv<T>& F, const Lv<T>& C) {
-    const T* __restrict__ e = C.dp;
-    T* __restrict__ d = F.dp;
+__device__ __forceinline__ void prolong(const Lv<T>& F, const Lv<T>& C, bool black_only) {
+    const T* __restrict__ e = C.dp;                   // (a coarse level's halves are one array)
+    T* __restrict__ dr = F.dp;
+    T* __restrict__ db = F.db;
     const int hx = F.hx, H = F.H;
+    if constexpr (Scaled<T>::value) {
+        if (black_only && wide<T, G>(hx, C.nc)) {     // two coarse cells a thread, 16-byte accesses
+            for (int c = 2 * G::rank(); c < C.nc; c += 2 * G::size()) {
+                const int J = fdiv(c, C.nx, C.mnx), I = c - J * C.nx, r0 = H + 2 * J * hx + I;
+                const double v0 = e[sidx(C, I, J)], v1 = e[sidx(C, I + 1, J)];
+                double a[2], b[2];
+                ld_vec(db + r0, a);
+                ld_vec(db + r0 + hx, b);
+                a[0] += v0; a[1] += v1; b[0] += v0; b[1] += v1;
+                st_vec(db + r0, a);
+                st_vec(db + r0 + hx, b);
+            }
+            G::sync();
+            return;
+        }
+    }
 #pragma unroll 2
     for (int c = G::rank(); c < C.nc; c += G::size()) {
         const int J = fdiv(c, C.nx, C.mnx), I = c - J * C.nx;
         const T v = e[sidx(C, I, J)];
         const int r0 = 2 * J * hx + I;
-        d[r0] += v; d[r0 + hx] += v; d[H + r0] += v; d[H + r0 + hx] += v;
+        db[H + r0] += v; db[H + r0 + hx] += v;
+        if (!black_only) { dr[r0] += v; dr[r0 + hx] += v; }
     }
     G::sync();
 }
 
-// exact coarsest solve: Gaussian elimination of the assembled five-point
-// matrix by one warp in shared memory (symmetric, diagonally dominant); run
-// by warp 0 only, synchronised with __syncwarp
+// Exact coarsest solve: Gaussian elimination of the assembled five-point
+// matrix (symmetric positive definite, diagonally dominant: no pivoting) in
+// shared memory.  The matrix is factored once per Picard iteration -- the upper
+// triangle, the row multipliers below it and the reciprocals of the pivots in
+// the extra column -- and a cycle's visit substitutes its right-hand side with
+// the same operations in the same order.  A visit then has no division: n
+// dependent FP64 divisions of about 560 cycles each for the pivots and as many
+// for the multipliers made it 5000 cycles on a 2^2 coarsest level; it is about
+// 1600 without them.  Run by warp 0.
 template <typename T>
-__device__ __forceinline__ void coarse_solve_warp(int nx, int nz, const T* Tx, const T* Tz, const T* D,
-                                                  const T* f, T* dp, T* A) {
+__device__ void coarse_factor_warp(int nx, int nz, const T* Tx, const T* Tz, const T* D, T* A) {
     const int nn = nx * nz, ld = nn + 1, lane = threadIdx.x & 31;
     for (int r = lane; r < nn; r += 32) {
         for (int c = 0; c < nn; ++c) A[r * ld + c] = T(0);
@@ -458,40 +619,64 @@ __device__ __forceinline__ void coarse_solve_warp(int nx, int nz, const T* Tx, c
         if (i > 0)      A[r * ld + r - 1] = -Tx[r - 1];
         if (j < nz - 1) A[r * ld + r + nx] = -Tz[r];
         if (j > 0)      A[r * ld + r - nx] = -Tz[r - nx];
-        A[r * ld + nn] = f[r];
     }
     __syncwarp();
     for (int k = 0; k < nn; ++k) {
         for (int r = k + 1 + lane; r < nn; r += 32) {
-            T m = A[r * ld + k] / A[k * ld + k];
-            for (int c = k; c <= nn; ++c) A[r * ld + c] -= m * A[k * ld + c];
+            const T m = A[r * ld + k] / A[k * ld + k];
+            A[r * ld + k] = m;
+            for (int c = k + 1; c < nn; ++c) A[r * ld + c] = fma(-m, A[k * ld + c], A[r * ld + c]);
         }
         __syncwarp();
     }
-    if (lane == 0) {
-        for (int k = nn - 1; k >= 0; --k) {
-            T sum = A[k * ld + nn];
-            for (int c = k + 1; c < nn; ++c) sum -= A[k * ld + c] * A[c * ld + nn];
-            A[k * ld + nn] = sum / A[k * ld + k];
-        }
-    }
-    __syncwarp();
-    for (int r = lane; r < nn; r += 32) dp[r] = A[r * ld + nn];
+    for (int r = lane; r < nn; r += 32) A[r * ld + nn] = T(1) / A[r * ld + r];
     __syncwarp();
 }
 
-// exact solve on the coarsest level c (FP64 levels: the unscaled FP64
-// operator; f0 is the unscaled right-hand side when c is the finest level),
-// by warp 0; the CTA group waits for it at a barrier
-template <typename T, typename G>
-__device__ __forceinline__ void coarsest(const Lv<T>* L, const Lv64* L64, int c, T* A, const T* f0) {
-    if (threadIdx.x < 32) {
-        if constexpr (Scaled<T>::value)
-            coarse_solve_warp<T>(L64[c].nx, L64[c].nz, L64[c].Tx, L64[c].Tz, L64[c].D, c == 0 ? f0 : L[c].f,
-                                 L[c].dp, A);
-        else
-            coarse_solve_warp<T>(L[c].nx, L[c].nz, L[c].c0, L[c].c1, L[c].D, L[c].f, L[c].dp, A);
+// s / u given r = 1/u rounded to nearest: the quotient s r corrected by its
+// exact remainder is the correctly rounded s / u (Markstein, IBM J. Res. Dev.
+// 34, 1990; tiny and huge operands, where the remainder may not be exact, and
+// a zero or non-finite pivot take the division)
+__device__ __forceinline__ double div_by(double s, double u, double r) {
+    const double q = s * r;
+    const int eq = (__double2hiint(q) >> 20 & 0x7FF) - 1023, eu = (__double2hiint(u) >> 20 & 0x7FF) - 1023;
+    if (abs(eq) < 600 && abs(eu) < 300) return fma(fma(-q, u, s), r, q);
+    return s / u;
+}
+__device__ __forceinline__ float div_by(float s, float u, float) { return s / u; }
+
+template <typename T>
+__device__ __forceinline__ void coarse_solve_warp(int nn, const T* f, T* dp, const T* A) {
+    const int ld = nn + 1, lane = threadIdx.x & 31;
+    // forward: lane r mod 32 owns row r (dp holds the eliminated right-hand side)
+    for (int r = lane; r < nn; r += 32) dp[r] = f[r];
+    __syncwarp();
+    if (nn <= 8) {                                    // a handful of rows: one lane, no exchanges
+        if (lane == 0) {
+            for (int k = 0; k < nn; ++k)
+                for (int r = k + 1; r < nn; ++r) dp[r] = fma(-A[r * ld + k], dp[k], dp[r]);
+        }
+    } else {
+        for (int k = 0; k < nn; ++k) {
+            for (int r = k + 1 + lane; r < nn; r += 32) dp[r] = fma(-A[r * ld + k], dp[k], dp[r]);
+            __syncwarp();
+        }
     }
+    if (lane == 0) {
+        for (int k = nn - 1; k >= 0; --k) {
+            T sum = dp[k];
+            for (int c = k + 1; c < nn; ++c) sum = fma(-A[k * ld + c], dp[c], sum);
+            dp[k] = div_by(sum, A[k * ld + k], A[k * ld + nn]);
+        }
+    }
+    __syncwarp();
+}
+
+// exact solve on the coarsest level c (f0 is the unscaled right-hand side when
+// c is the finest level), by warp 0; the CTA group waits for it at a barrier
+template <typename T, typename G>
+__device__ __forceinline__ void coarsest(const Lv<T>* L, int c, const T* A, const T* f0) {
+    if (threadIdx.x < 32) coarse_solve_warp<T>(L[c].nc, Scaled<T>::value && c == 0 ? f0 : L[c].f, L[c].dp, A);
     if constexpr (std::is_same<G, GCta>::value) __syncthreads();
 }
 
@@ -506,7 +691,7 @@ __device__ __forceinline__ void coarsest(const Lv<T>* L, const Lv64* L64, int c,
 // first red half-sweep, which the restriction seeded; a level cycled again
 // (gamma > 1) starts from its previous correction and smooths in full.
 template <typename T, typename G>
-__device__ __forceinline__ void gwalk(const Lv<T>* L, const Lv64* L64, int root, int nlev, int lw, int nu1, int nu2,
+__device__ __forceinline__ void gwalk(const Lv<T>* L, int root, int nlev, int lw, int nu1, int nu2,
                                       int gamma, T* A, const T* f0, bool root_fresh) {
     static_assert(RICH_MAX_LEVELS * 4 <= 64, "visit counters must fit one 64-bit word");
     unsigned long long cnt = 0;
@@ -523,13 +708,13 @@ __device__ __forceinline__ void gwalk(const Lv<T>* L, const Lv64* L64, int root,
         if constexpr (std::is_same<G, GCta>::value) {
             if (l == lw && lw < nlev - 1) {
                 if (threadIdx.x < 32)
-                    gwalk<T, GWarp>(L, L64, lw, nlev, nlev, nu1, nu2, gamma, A, f0, fresh && seed);
+                    gwalk<T, GWarp>(L, lw, nlev, nlev, nu1, nu2, gamma, A, f0, fresh && seed);
                 __syncthreads();
             } else {
-                coarsest<T, G>(L, L64, nlev - 1, A, f0);
+                coarsest<T, G>(L, nlev - 1, A, f0);
             }
         } else {
-            coarsest<T, G>(L, L64, nlev - 1, A, f0);
+            coarsest<T, G>(L, nlev - 1, A, f0);
         }
         for (;;) {                                        // leave l+1, back on l
             if (--l < root) return;
@@ -542,14 +727,15 @@ __device__ __forceinline__ void gwalk(const Lv<T>* L, const Lv64* L64, int root,
 }
 
 // V-cycle with the levels from lw down handed to warp 0 (lw = nlev: none);
-// every level below the finest is fresh (seeded by its restriction)
+// every level below the finest is fresh (seeded by its restriction), the
+// finest when `fresh`
 template <typename T>
-__device__ __forceinline__ void vcycle(const Lv<T>* L, const Lv64* L64, int nlev, int lw, int nu1, int nu2, T* A,
-                                       const T* f0) {
+__device__ __forceinline__ void vcycle(const Lv<T>* L, int nlev, int lw, int nu1, int nu2, T* A, const T* f0,
+                                       bool fresh) {
     const bool seed = nu1 > 0;
     const int top = min(lw, nlev - 1);       // levels 0 .. top-1 run on the whole CTA
     for (int l = 0; l < top; ++l) {
-        smooth<T, GCta>(L[l], nu1, l > 0 && seed);
+        smooth<T, GCta>(L[l], nu1, (l > 0 || fresh) && seed);
         resid_restrict<T, GCta>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
     }
     if (lw < nlev - 1) {
@@ -558,35 +744,67 @@ __device__ __forceinline__ void vcycle(const Lv<T>* L, const Lv64* L64, int nlev
                 smooth<T, GWarp>(L[l], nu1, seed);
                 resid_restrict<T, GWarp>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
             }
-            coarsest<T, GWarp>(L, L64, nlev - 1, A, f0);
+            coarsest<T, GWarp>(L, nlev - 1, A, f0);
             for (int l = nlev - 2; l >= lw; --l) prolong_smooth<T, GWarp>(L[l], L[l + 1], nu2);
         }
         __syncthreads();
     } else {
-        coarsest<T, GCta>(L, L64, nlev - 1, A, f0);
+        coarsest<T, GCta>(L, nlev - 1, A, f0);
     }
     for (int l = top - 1; l >= 0; --l) prolong_smooth<T, GCta>(L[l], L[l + 1], nu2);
 }
 
-// ||f - A dp||_inf on a level after a cycle ending with a black half-sweep
-// (red cells only) or, with red_only false, over every cell
+// ||f - A dp||_inf on the finest (FP64) level after a cycle ending with a black
+// half-sweep (red cells only) or, with red_only false, over every cell.  The
+// red cells' scaled residual is g - dp with g the value that the next red
+// half-sweep would store: with `next` given, g is kept there, and the next
+// cycle starts from that half (see Cta::mg_solve) instead of sweeping.
 template <typename T>
-__device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool red_only,
+__device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool red_only, T* __restrict__ next,
                                                          unsigned long long* red) {
+    static_assert(Scaled<T>::value, "the mixed path's norm is its FP64 defect's");
     unsigned long long m = 0;
-    if (red_only) {
-        const int n = L.hx * L.nz;
-#pragma unroll 2
-        for (int c = threadIdx.x; c < n; c += blockDim.x) {
-            const int j = fdiv(c, L.hx, L.mhx);
-            const int i = 2 * (c - j * L.hx) + (j & 1);
-            const unsigned long long b = abs_bits((double)resid_cell(L, i, j));
-            m = b > m ? b : m;
+    const int nx = L.nx, nz = L.nz, hx = L.hx, H = L.H;
+    if (H) {
+        for (int col = 0; col < (red_only ? 1 : 2); ++col) {
+            const T* __restrict__ own = col ? L.db : L.dp;
+            const T* __restrict__ oth = col ? L.dp : L.db;
+            const T* __restrict__ D = L.D;
+            if (wide<T, GCta>(hx, H)) {
+                for (int c = 2 * threadIdx.x; c < H; c += 2 * blockDim.x) {
+                    T g[2], d[2], x[2];
+                    gs_vec<T>(c, fdiv(c, hx, L.mhx), nz, hx, H, col, L.f, L.c0, L.c1, L.c2, L.c3, L.q, oth, g);
+                    ld_vec(D + col * H + c, d);
+                    ld_vec(own + col * H + c, x);
+                    if (next) st_vec(next + c, g);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const unsigned long long b = abs_bits(d[t] * (g[t] - x[t]));
+                        m = b > m ? b : m;
+                    }
+                }
+                continue;
+            }
+#pragma unroll 1
+            for (int c = threadIdx.x; c < H; c += blockDim.x) {
+                const int j = fdiv(c, hx, L.mhx);
+                const int i = 2 * (c - j * hx) + ((j + col) & 1);
+                const Nb s = nb_half(col, c, i, hx, H);
+                const T g = gs_at<T>(s, i < nx - 1, i > 0, j < nz - 1, j > 0, L.f, L.c0, L.c1, L.c2, L.c3, L.q, oth);
+                if (next) next[c] = g;
+                const unsigned long long b = abs_bits(D[s.own] * (g - own[s.own]));
+                m = b > m ? b : m;
+            }
         }
-    } else {
+    } else {                                          // one level only: natural order
         for (int c = threadIdx.x; c < L.nc; c += blockDim.x) {
-            const int j = fdiv(c, L.nx, L.mnx), i = c - j * L.nx;
-            const unsigned long long b = abs_bits((double)resid_cell(L, i, j));
+            const int j = fdiv(c, nx, L.mnx), i = c - j * nx;
+            T v = L.f[c];
+            if (i < nx - 1) v += L.c0[c] * L.dp[c + 1];
+            if (i > 0) v += L.c1[c] * L.dp[c - 1];
+            if (j < nz - 1) v += L.c2[c] * L.dp[c + nx];
+            if (j > 0) v += L.c3[c] * L.dp[c - nx];
+            const unsigned long long b = abs_bits(L.D[c] * (v - L.dp[c]));
             m = b > m ? b : m;
         }
     }
@@ -634,7 +852,7 @@ struct Cta {
     __device__ Cta(const FParams& P_, char* slot, Lv64* l64, Lv<TM>* lm, TM* A, unsigned long long* r)
         : P(P_), L64(l64), LM(lm), Amat(A), red(r) {
         f64 = (double*)(slot + P.o_f64);
-        dp64 = SC ? (double*)LM[0].dp : (double*)(slot + P.o_dp64);
+        dp64 = SC ? nullptr : (double*)(slot + P.o_dp64);
         p = (double*)(slot + P.o_p);
         thold = (double*)(slot + P.o_thold);
         Ks = (double*)(slot + P.o_Ks);
@@ -719,6 +937,14 @@ struct Cta {
         __syncthreads();
     }
 
+    // a cell's correction at the start of a solve on the finest level: zero, or
+    // (nu1 > 0) in red cells the value v = f/D that the first red half-sweep
+    // would give them, which the first cycle then skips
+    __device__ __forceinline__ void start_cell(const Lv<TM>& M0, int i, int j, TM v) const {
+        const bool black = (i + j) & 1;
+        (black && M0.H ? M0.db : M0.dp)[sidx(M0, i, j)] = black || !M0.H || P.nu1 == 0 ? TM(0) : v;
+    }
+
     // Picard system at p (Gardner closure, harmonic faces, f = -R), all levels;
     // returns ||f||_inf as a bit pattern
     __device__ unsigned long long assemble() {
@@ -774,17 +1000,20 @@ struct Cta {
             else { double t = F.Tbb[i]; R += t * (pp - P.p_bot) + t * h / 2.0; d += t; }
             F.D[q] = d;
             f64[q] = -R;
-            dp64[q] = 0.0;
             const int sq = sidx(M0, i, j);
             if constexpr (SC) {
                 double inv = 1.0 / d;
                 M0.q[sq] = inv; M0.D[sq] = d;
                 M0.c0[sq] = te * inv; M0.c1[sq] = tw * inv; M0.c2[sq] = tn * inv; M0.c3[sq] = tsf * inv;
                 M0.f[sq] = -R * inv;
+                start_cell(M0, i, j, -R * inv);
             } else {
+                const float qf = 1.0f / (float)d;
                 M0.c0[sq] = (TM)te; M0.c1[sq] = (TM)tn; M0.D[sq] = (TM)d;
-                M0.q[sq] = (TM)(1.0f / (float)d);
-                M0.f[sq] = (TM)(-R); M0.dp[q] = TM(0);
+                M0.q[sq] = (TM)qf;
+                M0.f[sq] = (TM)(-R);
+                dp64[q] = 0.0;
+                start_cell(M0, i, j, (TM)(-R) * (TM)qf);
             }
             unsigned long long b = abs_bits(R);
             m = b > m ? b : m;
@@ -811,7 +1040,7 @@ struct Cta {
                 const int sc = sidx(Ml, I, J);
                 if constexpr (SC) {
                     double inv = 1.0 / d;
-                    Ml.q[sc] = inv; Ml.D[sc] = d;
+                    Ml.q[sc] = 0.25 * inv; Ml.D[sc] = d;
                     Ml.c0[sc] = te * inv; Ml.c1[sc] = tw * inv; Ml.c2[sc] = tn * inv; Ml.c3[sc] = tsf * inv;
                 } else {
                     Ml.c0[sc] = (TM)te; Ml.c1[sc] = (TM)tn; Ml.D[sc] = (TM)d;
@@ -820,20 +1049,29 @@ struct Cta {
             }
             __syncthreads();
         }
+        if (tid < 32) {
+            const Lv64& Z = L64[nlev - 1];
+            const Lv<TM>& Mz = LM[nlev - 1];
+            if constexpr (SC) coarse_factor_warp<TM>(Z.nx, Z.nz, Z.Tx, Z.Tz, Z.D, Amat);
+            else coarse_factor_warp<TM>(Z.nx, Z.nz, Mz.c0, Mz.c1, Mz.D, Amat);
+        }
+        __syncthreads();
         return fb;
     }
 
     // one multigrid cycle: the V-cycle, or (WC, a separate kernel
     // instantiation so the V kernels keep their register allocation) the
     // cycle of index P.gamma
-    __device__ void mgcycle(const TM* f0) {
-        if constexpr (WC) gwalk<TM, GCta>(LM, L64, 0, nlev, P.lw, P.nu1, P.nu2, P.gamma, Amat, f0, false);
-        else vcycle<TM>(LM, L64, nlev, P.lw, P.nu1, P.nu2, Amat, f0);
+    // (fresh: the red cells already hold their first half-sweep's values)
+    __device__ void mgcycle(const TM* f0, bool fresh) {
+        if constexpr (WC) gwalk<TM, GCta>(LM, 0, nlev, P.lw, P.nu1, P.nu2, P.gamma, Amat, f0, fresh);
+        else vcycle<TM>(LM, nlev, P.lw, P.nu1, P.nu2, Amat, f0, fresh);
     }
 
     // x += e (FP64, natural order += FP32 finest-level correction), then the
     // CTA synchronises
     __device__ __forceinline__ void add_correction(double* __restrict__ x, const TM* __restrict__ e) const {
+        // (the mixed path's halves of dp never swap: e is one array)
         const Lv<TM>& M0 = LM[0];
         const unsigned mnx = L64[0].mnx;
 #pragma unroll 4
@@ -845,14 +1083,17 @@ struct Cta {
     }
 
     // FP64 defect r = f - A x of the finest operator, stored as the next FP32
-    // right-hand side rf (with the FP32 correction ef cleared); returns this
-    // thread's max |r| as a bit pattern (distinct arrays: restrict views)
+    // right-hand side rf (with the FP32 correction ef at its start values, see
+    // start_cell); returns this thread's max |r| as a bit pattern (distinct
+    // arrays: restrict views)
     __device__ __forceinline__ unsigned long long defect(const double* __restrict__ f, const double* __restrict__ x,
                                                          const double* __restrict__ Tx,
                                                          const double* __restrict__ Tz,
-                                                         const double* __restrict__ D, TM* __restrict__ rf,
+                                                         const double* __restrict__ D,
+                                                         const TM* __restrict__ qf, TM* __restrict__ rf,
                                                          TM* __restrict__ ef) const {
         const unsigned mnx = L64[0].mnx;
+        const bool seed = P.nu1 > 0 && nlev > 1;
         unsigned long long mm = 0;
 #pragma unroll 2
         for (int q = tid; q < nc; q += nt) {
@@ -865,7 +1106,7 @@ struct Cta {
             const double r = f[q] - (D[q] * x[q] - sn);
             const int sq = sidx(LM[0], i, j);
             rf[sq] = (TM)r;
-            ef[sq] = TM(0);
+            ef[sq] = seed && !((i + j) & 1) ? (TM)r * qf[sq] : TM(0);
             const unsigned long long b = abs_bits(r);
             mm = b > mm ? b : mm;
         }
@@ -881,24 +1122,43 @@ struct Cta {
         const double target = P.mg_tol * (fn > 1.0 ? fn : 1.0);
         double rn = fn;
         int cyc = 0;
+        // FP64: the stopping norm evaluates the next red half-sweep's values
+        // anyway; it stores them in the second red half, and a cycle that
+        // follows starts from that half (2 of about 30 FP64 instructions per
+        // cell and cycle).  The accepted correction keeps the old half.
+        const bool keep = SC && P.nu1 > 0 && P.nu2 > 0 && nlev > 1;
+        bool fresh = true;                            // assemble() seeded the red cells
         while (rn >= target && cyc < P.mg_maxit) {
             unsigned long long rb;
             if constexpr (SC) {
-                mgcycle((const TM*)f64);
+                if (cyc > 0) {
+                    if (keep) {
+                        if (tid == 0) { TM* t = LM[0].dp; LM[0].dp = LM[0].alt; LM[0].alt = t; }
+                        __syncthreads();
+                    }
+                    fresh = keep;
+                }
+                mgcycle((const TM*)f64, fresh);
                 ++cyc;
-                rb = resid_norm<TM>(M0, P.nu2 > 0 && nlev > 1, red);
+                rb = resid_norm<TM>(M0, P.nu2 > 0 && nlev > 1, keep ? M0.alt : nullptr, red);
             } else {
                 for (int in = 0; in < P.mixed_inner && cyc < P.mg_maxit; ++in) {
-                    mgcycle(nullptr);
+                    mgcycle(nullptr, in == 0);
                     ++cyc;
                 }
                 // dp += e in FP64, then the FP64 defect: stopping norm and the
                 // next FP32 right-hand side
                 add_correction(dp64, M0.dp);
-                rb = block_max(defect(f64, dp64, L64[0].Tx, L64[0].Tz, L64[0].D, M0.f, M0.dp), red);
+                rb = block_max(defect(f64, dp64, L64[0].Tx, L64[0].Tz, L64[0].D, M0.q, M0.f, M0.dp), red);
             }
             if (rb > INF_BITS - 1) { mg_tot += cyc; return false; }
             rn = __longlong_as_double((long long)rb);
+        }
+        if constexpr (SC) {
+            if (cyc == 0) {                           // nothing to solve: the correction is zero, not its seed
+                for (int c = tid; c < M0.H; c += nt) M0.dp[c] = TM(0);
+                __syncthreads();
+            }
         }
         mg_tot += cyc;
         if (!(rn < target)) status = max(status, (int)RICH_MG_MAXIT);
@@ -922,7 +1182,7 @@ struct Cta {
                 double d;
                 if constexpr (SC) {
                     const int j = fdiv(q, nx, L64[0].mnx);
-                    d = dp64[sidx(LM[0], q - j * nx, j)];
+                    d = dp_at(LM[0], q - j * nx, j);
                 } else {
                     d = dp64[q];
                 }
@@ -994,19 +1254,20 @@ struct Cta {
     }
 
     // approximate e = A^{-1} r by ninner V-cycles from e = 0 (A: the Picard
-    // operator assembled at the same state); e is returned in dp64 / M0.dp
+    // operator assembled at the same state); e is returned in the finest
+    // level's dp
     __device__ void mg_apply(const double* r, int ninner) {
         const Lv<TM>& M0 = LM[0];
         for (int q = tid; q < nc; q += nt) {
             const int j = fdiv(q, nx, L64[0].mnx), sq = sidx(M0, q - j * nx, j);
-            if constexpr (SC) M0.f[sq] = r[q] * M0.q[sq];
-            else M0.f[sq] = (TM)r[q];
-            M0.dp[q] = TM(0);
+            const TM v = (TM)r[q] * M0.q[sq];
+            M0.f[sq] = SC ? v : (TM)r[q];
+            start_cell(M0, q - j * nx, j, v);
         }
         __syncthreads();
         for (int k = 0; k < ninner; ++k) {
-            if constexpr (SC) mgcycle(r);
-            else mgcycle(nullptr);
+            if constexpr (SC) mgcycle(r, k == 0);
+            else mgcycle(nullptr, k == 0);
         }
     }
 
@@ -1030,7 +1291,7 @@ struct Cta {
             mg_apply(r, P.adj_inner);
             for (int q = tid; q < nc; q += nt) {
                 const int j = fdiv(q, nx, L64[0].mnx);
-                lam[q] += (double)M0.dp[sidx(M0, q - j * nx, j)];
+                lam[q] += (double)dp_at(M0, q - j * nx, j);
             }
             __syncthreads();
             unsigned long long mm = 0;
@@ -1051,10 +1312,9 @@ struct Cta {
     // linear operator: the same cycles on the same matrix), copied to out
     __device__ void precond(const double* r, double* out) {
         mg_apply(r, P.adj_inner);
-        const TM* e = LM[0].dp;
         for (int q = tid; q < nc; q += nt) {
-            const int j = fdiv(q, nx, L64[0].mnx), sq = sidx(LM[0], q - j * nx, j);
-            out[q] = (double)e[sq];
+            const int j = fdiv(q, nx, L64[0].mnx);
+            out[q] = (double)dp_at(LM[0], q - j * nx, j);
         }
         __syncthreads();
     }
@@ -1322,11 +1582,13 @@ __device__ __forceinline__ void init_levels(const FParams& P, char* slot, unsign
         Lv<TM>& b = LM[l];
         b.nx = a.nx; b.nz = a.nz; b.hx = a.nx >> 1; b.nc = a.nc; b.mnx = P.mnx[l]; b.mhx = P.mhx[l];
         b.H = l < nlev - 1 ? b.hx * b.nz : 0;             // colour-split unless coarsest
-        TM** qq[NMG] = {&b.c0, &b.c1, &b.c2, &b.c3, &b.q, &b.f, &b.dp, &b.D};
+        TM** qq[NMG] = {&b.c0, &b.c1, &b.c2, &b.c3, &b.q, &b.f, &b.dp, &b.D, &b.alt};
         for (int k = 0; k < NMG; ++k)
             *qq[k] = P.smg[l][k] >= 0 ? (TM*)(sm + P.smg[l][k])
                    : P.omg[l][k] >= 0 ? (TM*)(slot + P.omg[l][k]) : nullptr;
         if (P.osm[l] >= 0) b.dp = (TM*)(sm + P.osm[l]);   // corrections of small levels on chip
+        if (l == 0 && P.osm_alt >= 0) b.alt = (TM*)(sm + P.osm_alt);
+        b.db = b.dp;
         if constexpr (!SC) { b.D = b.c3; b.c3 = nullptr; }   // FP32: D in the c3 slot
     }
     __syncthreads();
