@@ -91,10 +91,9 @@ static int fused_setup(const rich_problem_t* pb, int S, FParams& P, int ckpt_eve
             P.o64[l][k] = (long long)off; off = al256(off + bytes);
         }
         for (int k = 0; k < NMG; ++k) {
-            // FP64: wE wW wN wS q f dp D alt (the half array alt on the finest level
-            // only); FP32: Tx Tz - D q f dp - -
-            if (mixed ? (k == B_2 || k == B_7 || k == B_ALT) : (l > 0 && k == B_ALT)) { P.omg[l][k] = -1; continue; }
-            P.omg[l][k] = (long long)off; off = al256(off + (k == B_ALT ? (nc + 1) / 2 : nc) * w);
+            // FP64: wE wW wN wS q f dp D ; FP32: Tx Tz - D q f dp - (slots B_2, B_7 unused)
+            if (mixed && (k == B_2 || k == B_7)) { P.omg[l][k] = -1; continue; }
+            P.omg[l][k] = (long long)off; off = al256(off + nc * w);
         }
         lx /= 2; lz /= 2;
     }
@@ -159,6 +158,31 @@ static int fused_launch(const FParams& P, int grid, size_t smem, int nt, cudaStr
     return 0;
 }
 
+// Threads per CTA when the caller has not chosen them (rich_set_tuning 0).  A
+// CTA runs one sample: too many threads leave a small grid's levels with idle
+// warps at every barrier and too few samples on an SM; too few leave a large
+// grid's loads exposed.  Where the lines lie (ms of a batch on GB300, FP64
+// Gardner unless stated, 32 / 128 / 256 / 512 / 1024 threads):
+//   8^2   x 8192:  18 / 24 / 37 / 72 / 150       16^2 x 1216: 18 / 13 / 16 / 24 / 43
+//   16^2  x 8192:  60 / 64 / 81 / 135 / 264      32^2 x 1:    28 / 11 / 9.3 / 9.3 / 9.7
+//   32^2  x 4864:  193 / 141 / 151 / 211 / 345   32^2 x 608:  68 / 33 / 31 / 36 / 53
+//   48x40 x 2048:  281 / 185 / 179 / 237 / 365   48x40 x 152: 201 / 93 / 77 / 74 / 74
+//   64^2  x 1216:  - / 268 / 203 / 190 / 257     64^2 x 1:    - / 33 / 23 / 22 / 23
+//   128^2 x 608:   - / 457 / 304 / 296 / 325     128^2 x 304: - / 293 / 193 / 166 / 144
+//   256^2 x 152:   - / - / 610 / 409 / 350
+// Mixed precision and the van Genuchten closure rank the shapes alike.
+static int default_threads(long long nc, int S, int sms) {
+    const long long per_sm = (S + sms - 1) / std::max(sms, 1);
+    if (nc <= 64) return per_sm > 16 ? 32 : 128;
+    if (nc <= 256) return 128;
+    if (nc <= 1024) return per_sm > 16 ? 128 : 256;
+    if (nc <= 2048) return per_sm > 8 ? 256 : 512;
+    if (nc <= 8192) return 512;
+    // one 1024-thread CTA per SM keeps more of a large grid in L2 and on chip;
+    // two 512-thread CTAs overlap better once the batch fills the GPU twice
+    return nc > 32768 || per_sm <= 2 ? 1024 : 512;
+}
+
 // Fused persistent solve of S samples; stats arrays live in ctx->ws, the
 // per-CTA slots and the queue counter in ctx->fused_scratch.
 int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const double* lnKs,
@@ -168,8 +192,8 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     FParams P;
     if (pb->closure == RICH_VAN_GENUCHTEN && (!soil || !soil->n)) return RICH_ERR_INVALID;
     const int nt = (ctx->tune_threads == 1024 || ctx->tune_threads == 256 || ctx->tune_threads == 128 ||
-                    ctx->tune_threads == 32)
-                       ? ctx->tune_threads : 512;
+                    ctx->tune_threads == 32 || ctx->tune_threads == 512)
+                       ? ctx->tune_threads : default_threads((long long)pb->nx * pb->nz, S, ctx->sm_count);
     if (int e = fused_setup(pb, S, P)) return e;
     plan_smem(P, nt);
     if (soil) {

@@ -52,9 +52,8 @@ constexpr int ADJ_M = 12;                // GMRES restart length of the adjoint'
 // FP64 unscaled operator (all levels): faces, mass term, diagonal, Dirichlet faces
 enum { A_TX, A_TZ, A_CDT, A_D, A_TBT, A_TBB, N64 };
 // multigrid arrays in the cycle precision, colour-split on every level but
-// the coarsest.  FP64: wE wW wN wS q=1/D fh dp D alt (the second red half alt
-// of dp on the finest level only).  FP32: Tx Tz - D 1/D f dp - -.
-enum { B_0, B_1, B_2, B_3, B_4, B_5, B_6, B_7, B_ALT, NMG };
+// the coarsest.  FP64: wE wW wN wS q=1/D fh dp D.  FP32: Tx Tz - D 1/D f dp -.
+enum { B_0, B_1, B_2, B_3, B_4, B_5, B_6, B_7, NMG };
 
 struct FParams {
     int S, nlev, mixed;
@@ -998,7 +997,7 @@ struct Cta {
             else { double t = F.Tbt[i]; R += -t * (P.p_top - pp) - t * h / 2.0; d += t; }
             if (j > 0)      { tsf = F.Tz[q - nx]; R += -tsf * (p[q - nx] - pp) + tsf * h; d += tsf; }
             else { double t = F.Tbb[i]; R += t * (pp - P.p_bot) + t * h / 2.0; d += t; }
-            F.D[q] = d;
+            if (!SC || nlev == 1) F.D[q] = d;     // read by the defect, or the only level's factorisation
             f64[q] = -R;
             const int sq = sidx(M0, i, j);
             if constexpr (SC) {
@@ -1036,7 +1035,8 @@ struct Cta {
                 else d += Cl.Tbt[I];
                 if (J > 0)         { tsf = 0.25 * (0.5 * (Fl.Tz[f00 - fx] + Fl.Tz[f00 - fx + 1])); d += tsf; }
                 else d += Cl.Tbb[I];
-                Cl.Tx[c] = te; Cl.Tz[c] = tn; Cl.Cdt[c] = cd; Cl.D[c] = d;
+                Cl.Tx[c] = te; Cl.Tz[c] = tn; Cl.Cdt[c] = cd;
+                if (SC && l == nlev - 1) Cl.D[c] = d;
                 const int sc = sidx(Ml, I, J);
                 if constexpr (SC) {
                     double inv = 1.0 / d;
@@ -1582,12 +1582,14 @@ __device__ __forceinline__ void init_levels(const FParams& P, char* slot, unsign
         Lv<TM>& b = LM[l];
         b.nx = a.nx; b.nz = a.nz; b.hx = a.nx >> 1; b.nc = a.nc; b.mnx = P.mnx[l]; b.mhx = P.mhx[l];
         b.H = l < nlev - 1 ? b.hx * b.nz : 0;             // colour-split unless coarsest
-        TM** qq[NMG] = {&b.c0, &b.c1, &b.c2, &b.c3, &b.q, &b.f, &b.dp, &b.D, &b.alt};
+        TM** qq[NMG] = {&b.c0, &b.c1, &b.c2, &b.c3, &b.q, &b.f, &b.dp, &b.D};
         for (int k = 0; k < NMG; ++k)
             *qq[k] = P.smg[l][k] >= 0 ? (TM*)(sm + P.smg[l][k])
                    : P.omg[l][k] >= 0 ? (TM*)(slot + P.omg[l][k]) : nullptr;
         if (P.osm[l] >= 0) b.dp = (TM*)(sm + P.osm[l]);   // corrections of small levels on chip
-        if (l == 0 && P.osm_alt >= 0) b.alt = (TM*)(sm + P.osm_alt);
+        // the second red half: on chip beside dp, else the natural-order diagonal's
+        // place in the slot (the FP64 cycles read their own copy of it)
+        b.alt = l > 0 || !SC ? nullptr : P.osm_alt >= 0 ? (TM*)(sm + P.osm_alt) : (TM*)a.D;
         b.db = b.dp;
         if constexpr (!SC) { b.D = b.c3; b.c3 = nullptr; }   // FP32: D in the c3 slot
     }
