@@ -381,7 +381,8 @@ int rich_kl_fields(rich_ctx_t ctx, const double* kl_basis, int32_t n_kl, int32_t
  * J^T systems are solved by BiCGStab (or defect correction, see
  * rich_set_adjoint_method) preconditioned with CCMG V-cycles of the Picard
  * operator (FP32 V-cycles when pb->precision is RICH_MIXED) to a relative
- * residual of 1e-11.  Memory: the states are checkpointed every
+ * residual of 1e-11.  Memory: the states of all steps are kept while those of
+ * the resident samples fit in 4 GiB; else they are checkpointed every
  * ckpt_every steps and each segment is recomputed during the reverse sweep.
  * dq_dlnKs [S][nz][nx] (device) may be NULL.  A J^T solve that stops at its
  * iteration limit sets RICH_MG_MAXIT.  Synchronous (returns when done). */

@@ -72,7 +72,7 @@ static void plan_smem(FParams& P, int nt) {
     P.smem_bytes = (long long)off;
 }
 
-static int fused_setup(const rich_problem_t* pb, int S, FParams& P, int ckpt_every = 0) {
+static int fused_setup(const rich_problem_t* pb, int S, FParams& P, int ckpt_every = 0, bool keep_states = false) {
     P = FParams{};
     const int nlev = rich_count_levels(pb->nx, pb->nz);
     if (nlev < 1) return RICH_ERR_INVALID;
@@ -116,8 +116,9 @@ static int fused_setup(const rich_problem_t* pb, int S, FParams& P, int ckpt_eve
     if (ckpt_every > 0) {
         const int nck = (pb->nsteps + ckpt_every - 1) / ckpt_every;
         P.ckpt_every = ckpt_every;
-        P.o_ckpt = off; off = al256(off + nc8 * std::max(nck, 1));
-        P.o_seg = off; off = al256(off + nc8 * ckpt_every);
+        P.keep_states = keep_states;
+        P.o_ckpt = off; off = al256(off + (keep_states ? 0 : nc8 * std::max(nck, 1)));
+        P.o_seg = off; off = al256(off + nc8 * (keep_states ? std::max(pb->nsteps, 1) : ckpt_every));
         long long* adj[] = {&P.o_lam, &P.o_rhs, &P.o_r, &P.o_dE, &P.o_dW, &P.o_dN, &P.o_dS, &P.o_dg, &P.o_g,
                             &P.o_rh, &P.o_pk, &P.o_v, &P.o_t, &P.o_ph, &P.o_sh};
         for (long long* o : adj) { *o = (long long)off; off = al256(off + nc8); }
@@ -231,6 +232,11 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     return 0;
 }
 
+// Device memory that the adjoint may use to keep the states of every time step
+// of its resident samples (1.5 % of the GPU's; 152 CTAs of a 256^2 grid keep 50
+// steps in it).  Within it nothing is recomputed and ckpt_every does not matter.
+constexpr size_t KEEP_STATES_BYTES = 4ull << 30;
+
 // Discrete adjoint of S samples: QoI and dQ/d ln Ks [S][nz][nx] (g_out).
 int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const double* lnKs,
                        const double* alpha, double alpha_scale, int ckpt_every, double adj_tol,
@@ -238,26 +244,32 @@ int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const dou
     rich_samplebuf& w = ctx->sb;
     FParams P;
     if (ckpt_every < 1 || pb->closure != RICH_GARDNER) return RICH_ERR_INVALID;
-    if (int e = fused_setup(pb, S, P, ckpt_every)) return e;
-    plan_smem(P, 512);
-    P.adj_tol = adj_tol; P.adj_maxit = adj_maxit; P.adj_inner = pb->precision == RICH_MIXED ? 2 : 1;
-    P.adj_method = adj_method;
-    P.mixed_inner = ctx->tune_mixed_inner > 0 ? ctx->tune_mixed_inner : MIXED_INNER_DEFAULT;
-    const size_t smem = fused_smem(P);
-    int occ = 0;
-    const void* kern = P.mixed ? rich_adjoint_kernel32(P.gamma > 1) : rich_adjoint_kernel64(P.gamma > 1);
-    if (int e = allow_dyn_smem(kern, smem)) return e;
-    RICH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 512, smem));
-    occ = std::max(occ, 1);
-    const int grid = std::max(1, std::min(S, ctx->sm_count * occ));
-    const size_t need = (size_t)grid * (size_t)P.slot_bytes + 256;
-    if (ctx->fused_bytes < need) {
+    size_t smem = 0;
+    int grid = 0;
+    for (bool keep : {true, false}) {
+        if (int e = fused_setup(pb, S, P, ckpt_every, keep)) return e;
+        plan_smem(P, 512);
+        smem = fused_smem(P);
+        int occ = 0;
+        const void* kern = P.mixed ? rich_adjoint_kernel32(P.gamma > 1) : rich_adjoint_kernel64(P.gamma > 1);
+        if (int e = allow_dyn_smem(kern, smem)) return e;
+        RICH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 512, smem));
+        occ = std::max(occ, 1);
+        grid = std::max(1, std::min(S, ctx->sm_count * occ));
+        if (keep && (size_t)grid * pb->nsteps * pb->nx * pb->nz * 8 > KEEP_STATES_BYTES) continue;
+        const size_t need = (size_t)grid * (size_t)P.slot_bytes + 256;
+        if (ctx->fused_bytes >= need) break;
         if (ctx->fused_scratch) cudaFree(ctx->fused_scratch);
         ctx->fused_scratch = nullptr; ctx->fused_bytes = 0;
         cudaError_t e = cudaMalloc(&ctx->fused_scratch, need);
-        if (e != cudaSuccess) { cudaGetLastError(); return RICH_ERR_OOM; }
-        ctx->fused_bytes = need;
+        if (e == cudaSuccess) { ctx->fused_bytes = need; break; }
+        cudaGetLastError();
+        ctx->fused_scratch = nullptr;
+        if (!keep) return RICH_ERR_OOM;               // the checkpointed layout needs less
     }
+    P.adj_tol = adj_tol; P.adj_maxit = adj_maxit; P.adj_inner = pb->precision == RICH_MIXED ? 2 : 1;
+    P.adj_method = adj_method;
+    P.mixed_inner = ctx->tune_mixed_inner > 0 ? ctx->tune_mixed_inner : MIXED_INNER_DEFAULT;
     P.scratch = (char*)ctx->fused_scratch + 256;
     P.queue = (int*)ctx->fused_scratch;
     P.lnKs = lnKs; P.alpha = alpha; P.alpha_scale = alpha_scale;

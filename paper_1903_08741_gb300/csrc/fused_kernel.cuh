@@ -86,7 +86,7 @@ struct FParams {
     double inv_dt, tr, ts, p_top, p_bot, p_init, picard_tol, mg_tol, h, two_over_h2;
     // adjoint (k_adjoint only)
     int mixed_inner;            // FP32 V-cycles per FP64 defect (mixed path)
-    int ckpt_every, adj_maxit, adj_inner;
+    int ckpt_every, keep_states, adj_maxit, adj_inner;
     double adj_tol;
     long long o_ckpt, o_seg, o_lam, o_rhs, o_r, o_dE, o_dW, o_dN, o_dS, o_dg, o_g;
     int adj_method;             // J^T solver: 0 defect correction, 1 BiCGStab, 2 GMRES(ADJ_M)
