@@ -123,7 +123,7 @@ extern "C" void rich_destroy(rich_ctx_t ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->sb.base) cudaFree(ctx->sb.base);
     if (ctx->stage) cudaFree(ctx->stage);
-    for (auto& e : ctx->spectra) { cudaFree(e.sq); cudaFree(e.tw); }
+    for (auto& e : ctx->spectra) cudaFree(e.tab);
     if (ctx->field_work) cudaFree(ctx->field_work);
     for (auto e : ctx->prof.ev) cudaEventDestroy(e);
     if (ctx->fused_scratch) cudaFree(ctx->fused_scratch);

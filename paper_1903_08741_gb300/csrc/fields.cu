@@ -4,18 +4,27 @@
 //
 // GPU design: the two real fields of a sample are packed into one complex
 // transform (re = y_0, im = y_1); sqrt(F c) is real and even, so the filter maps
-// real inputs to real outputs and the two fields come back in re / im.  The 2-D
-// FFT is two passes of batched 1-D radix-2 transforms in shared memory (rows,
-// then groups of adjacent columns so that global accesses stay coalesced).
+// real inputs to real outputs and the two fields come back in re / im.  Three
+// kernels, one pass over the torus each, in 64-bit integers (fixed.cuh has why
+// and how precise): white noise and row transforms; column transforms, filter
+// and inverse column transforms; inverse row transforms and the marginal
+// transforms.  The second keeps the rows of the physical window only, so the
+// third runs half of them.  Within the transforms frequencies stay in
+// bit-reversed order; the filter is laid out in it.  In FP64, one kernel a pass
+// (noise, row and column transforms both ways, filter, window), 512 draws of a
+// 128^2 pair took 63.1 ms, now 9.4; 64 of a 32^2 pair 477 us, now 103; 512
+// couples of five 64^2 fields 13.1 ms, now 3.7.
 // White noise: Philox4x32-10 (Salmon et al., SC'11) implemented from its
 // definition, key = (seed low word, seed high word ^ level), counter = (cell
 // pair, field, sample low, sample high), two uniforms -> Box-Muller.
 #include "rich_internal.cuh"
-#include <math.h>
+#include "fixed.cuh"
+#include <cmath>
 #include <vector>
 #include <algorithm>
 
 namespace {
+using namespace rich_fx;
 
 struct cplx { double re, im; };
 
@@ -30,40 +39,7 @@ __device__ __forceinline__ void philox10(uint32_t c[4], uint32_t k0, uint32_t k1
     }
 }
 
-__device__ __forceinline__ double u01(uint32_t hi, uint32_t lo) {
-    unsigned long long m = (((unsigned long long)hi << 32) | lo) >> 11;
-    return ((double)m + 0.5) * (1.0 / 9007199254740992.0);
-}
-
-// packed complex white noise: re = field fld0, im = field fld0 + 1, for
-// samples first..first+S-1 on the torus (npts = px*pz, even)
-// (first sample = *first_dev + first when first_dev is given: a captured CUDA
-// graph can advance the sample range between replays)
-__global__ void k_noise(int S, int npts, uint64_t seed, uint32_t level, int64_t first,
-                        const int64_t* __restrict__ first_dev, cplx* out, uint32_t fld0 = 0) {
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // (sample, pair)
-    const int pairs = npts >> 1;
-    if (g >= (long long)S * pairs) return;
-    int s = (int)(g / pairs), q = (int)(g - (long long)s * pairs);
-    uint64_t sample = (uint64_t)((first_dev ? *first_dev : 0) + first + s);
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32) ^ level;
-    double y[2][2];
-#pragma unroll
-    for (int fld = 0; fld < 2; ++fld) {
-        uint32_t c[4] = {(uint32_t)q, fld0 + (uint32_t)fld, (uint32_t)sample, (uint32_t)(sample >> 32)};
-        philox10(c, k0, k1);
-        double a = u01(c[0], c[1]), b = u01(c[2], c[3]);
-        double r = sqrt(-2.0 * log(a));
-        double sn, cs;
-        sincos(6.283185307179586476925286766559 * b, &sn, &cs);
-        y[fld][0] = r * cs; y[fld][1] = r * sn;
-    }
-    cplx* o = out + (size_t)s * npts + 2 * (size_t)q;
-    o[0] = cplx{y[0][0], y[1][0]};
-    o[1] = cplx{y[0][1], y[1][1]};
-}
-
-// twiddles w_k = exp(-2 pi i k / n), k < n/2
+// FP64 twiddles w_k = exp(-2 pi i k / n), k < n/2, of the spectrum's transform
 __global__ void k_twiddles(int n, cplx* tw) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n / 2) return;
@@ -72,14 +48,14 @@ __global__ void k_twiddles(int n, cplx* tw) {
     tw[k] = cplx{c, s};
 }
 
-// Batched radix-2 FFT of lines of length n (power of two) held in shared
-// memory.  A block handles LPB lines; line l of sample b starts at
+// Batched radix-2 FP64 FFT of lines of length n (power of two) held in shared
+// memory: the covariance spectrum's, once per model and grid (its values span
+// more than one fixed-point scale holds).  A block handles LPB lines; line l of sample b starts at
 // b*sample_stride + l*line_stride, its elements are elem_stride apart.
-// Bit-reversed load, log2(n) butterfly stages, 1/n on the inverse.
+// Bit-reversed load, log2(n) butterfly stages.
 template <int LPB>
 __global__ void k_fft_lines(cplx* data, int n, int logn, int lines, long long sample_stride,
-                            int line_stride, int elem_stride, const cplx* __restrict__ tw,
-                            int inverse) {
+                            int line_stride, int elem_stride, const cplx* __restrict__ tw) {
     // contiguous lines: consecutive threads take consecutive elements; strided
     // lines (columns): consecutive threads take adjacent lines
     const bool contig = elem_stride == 1;
@@ -96,14 +72,13 @@ __global__ void k_fft_lines(cplx* data, int n, int logn, int lines, long long sa
         sh[l * n + r] = base[(size_t)l * line_stride + (size_t)e * elem_stride];
     }
     __syncthreads();
-    const double sgn = inverse ? -1.0 : 1.0;
     for (int m = 1, st = n >> 1; m < n; m <<= 1, st >>= 1) {
         for (int t = tid; t < (n >> 1) * LPB; t += nt) {
             int l = t / (n >> 1), bf = t - l * (n >> 1);
             int grp = bf / m, k = bf - grp * m;
             int a = grp * 2 * m + k, c = a + m;
             cplx w = tw[k * st];
-            double wi = sgn * w.im;
+            double wi = w.im;
             cplx x = sh[l * n + c], y = sh[l * n + a];
             double xr = x.re * w.re - x.im * wi;
             double xi = x.re * wi + x.im * w.re;
@@ -112,20 +87,10 @@ __global__ void k_fft_lines(cplx* data, int n, int logn, int lines, long long sa
         }
         __syncthreads();
     }
-    const double sc = inverse ? 1.0 / (double)n : 1.0;
     for (int t = tid; t < n * LPB; t += nt) {
         int l = contig ? t / n : t % LPB, e = contig ? t - (t / n) * n : t / LPB;
-        cplx v = sh[l * n + e];
-        if (inverse) { v.re *= sc; v.im *= sc; }
-        base[(size_t)l * line_stride + (size_t)e * elem_stride] = v;
+        base[(size_t)l * line_stride + (size_t)e * elem_stride] = sh[l * n + e];
     }
-}
-
-__global__ void k_filter(int S, int npts, const double* __restrict__ sq, cplx* d) {
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long long)S * npts) return;
-    double w = sq[g % npts];
-    d[g].re *= w; d[g].im *= w;
 }
 
 // covariance model of one spectrum: nu = 0 exponential sigma2 exp(-r);
@@ -170,11 +135,17 @@ __global__ void k_cov(int px, int pz, double h, CovModel cm, cplx* c) {
     c[g] = cplx{v, 0.0};
 }
 
-__global__ void k_sqrt_spec(int npts, const cplx* __restrict__ lam, double* sq) {
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= npts) return;
-    double v = lam[g].re;
-    sq[g] = v > 0.0 ? sqrt(v) : 0.0;
+__device__ __forceinline__ int brev(int p, int logn) { return logn ? (int)(__brev((unsigned)p) >> (32 - logn)) : 0; }
+
+// the filter sqrt(max(F c, 0)) in Q62 of each column's scale 2^ecol, both
+// indices bit-reversed
+__global__ void k_filter_table(int logpx, int logpz, const cplx* __restrict__ lam, const int* __restrict__ ecol,
+                               wq* out) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >> (logpx + logpz)) return;
+    const int kx = brev(g & ((1 << logpx) - 1), logpx), kz = brev(g >> logpx, logpz);
+    const double v = lam[(kz << logpx) + kx].re;
+    out[g] = split_w(v > 0.0 ? __double2ll_rn(ldexp(sqrt(v), 62 - ecol[kx])) : 0);
 }
 
 // marginal transforms of a packed pair: the re lane is Gaussian (shift + z,
@@ -191,18 +162,202 @@ __device__ __forceinline__ double uniform_of(double z, double inv_sigma, double 
     return lo + span * 0.5 * erfc(-gg / sqrt(2.0));
 }
 
-// window of the torus -> the pair's two fields, in place into a compact
-// [S][nz][nx] pair of real arrays (al may be null: the im lane is unused)
-__global__ void k_window(int S, int nx, int nz, int px, int pz, const cplx* __restrict__ d,
-                         double inv_sigma, PackTr tr, double* lk, double* al) {
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int nc = nx * nz;
-    if (g >= (long long)S * nc) return;
-    int s = (int)(g / nc), q = (int)(g - (long long)s * nc);
-    int j = q / nx, i = q - j * nx;
-    cplx v = d[(size_t)s * px * pz + (size_t)j * px + i];
-    lk[g] = tr.re_uniform ? uniform_of(v.re, inv_sigma, tr.re_a, tr.re_b) : v.re + tr.re_a;
-    if (al) al[g] = uniform_of(v.im, inv_sigma, tr.im_lo, tr.im_span);
+// ---------------------------------------------------------------- transforms
+// One radix-R pass over the block's lines in shared memory, from bit b0 of the
+// n = 2^logn transform on.  Rows (COLS false) lie one after the other, an element
+// of padding after every eight: the last passes' strides of 4 and 8 elements then
+// meet no bank twice.  Columns lie side by side, LPB = 2^loglpb to a torus row.
+// With FILT (the last pass) each value is multiplied by its filter entry and the
+// first inverse pass follows in registers.
+template <bool COLS>
+__device__ __forceinline__ int at(int l, int p, int logn, int loglpb) {
+    return COLS ? (p << loglpb) + l : l * ((1 << logn) + ((1 << logn) >> 3)) + p + (p >> 3);
+}
+
+template <int R, bool COLS, bool INV, bool FILT>
+__device__ __forceinline__ void pass(fx2* sm, int logn, int loglpb, int b0, const cw* __restrict__ tw,
+                                     const wq* __restrict__ filt, int fstride) {
+    constexpr int RB = R == 8 ? 3 : R == 4 ? 2 : 1;
+    const int lq = logn - b0 - RB;                    // log2 of the stride between a butterfly's elements
+    const int sh = ((b0 + RB) >> 1) - (b0 >> 1);
+    for (int it = threadIdx.x; it < 1 << (logn - RB + loglpb); it += blockDim.x) {
+        const int l = COLS ? it & ((1 << loglpb) - 1) : it >> (logn - RB);
+        const int g = COLS ? it >> loglpb : it & ((1 << (logn - RB)) - 1);
+        const int k = g & ((1 << lq) - 1), base = ((g >> lq) << (lq + RB)) + k;
+        fx2 a[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) a[j] = sm[at<COLS>(l, base + (j << lq), logn, loglpb)];
+        if (FILT) {
+            dft_fwd<R>(a);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                const wq f = filt[(size_t)(base + j) * fstride + l];
+                a[j] = fx2{rmul(rshift(a[j].re, sh), f), rmul(rshift(a[j].im, sh), f)};
+            }
+            dft_inv<R>(a);
+        } else if (!INV) {
+            dft_fwd<R>(a);
+            a[0] = fx2{rshift(a[0].re, sh), rshift(a[0].im, sh)};
+#pragma unroll
+            for (int j = 1; j < R; ++j) a[j] = cmul(a[j], tw[(k * revr<R>(j)) << b0], sh);
+        } else {
+            if (lq > 0) {
+#pragma unroll
+                for (int j = 1; j < R; ++j) {
+                    cw w = tw[(k * revr<R>(j)) << b0];
+                    w.im = neg(w.im);
+                    a[j] = cmul(a[j], w, 0);
+                }
+            }
+            dft_inv<R>(a);
+        }
+#pragma unroll
+        for (int j = 0; j < R; ++j) sm[at<COLS>(l, base + (j << lq), logn, loglpb)] = a[j];
+    }
+    __syncthreads();
+}
+
+template <bool COLS, bool INV, bool FILT>
+__device__ __forceinline__ void any_pass(int bits, fx2* sm, int logn, int loglpb, int b0, const cw* tw,
+                                         const wq* filt = nullptr, int fstride = 0) {
+    if (bits == 3) pass<8, COLS, INV, FILT>(sm, logn, loglpb, b0, tw, filt, fstride);
+    else if (bits == 2) pass<4, COLS, INV, FILT>(sm, logn, loglpb, b0, tw, filt, fstride);
+    else pass<2, COLS, INV, FILT>(sm, logn, loglpb, b0, tw, filt, fstride);
+}
+
+// inverse passes below bit `top` (the passes of the forward order, last first)
+template <bool COLS>
+__device__ __forceinline__ void inverse_passes(fx2* sm, int logn, int loglpb, int top, const cw* tw) {
+    int b0s[8], np = 0;
+    for (int b = 0; b < top; b += pass_bits(logn, b)) b0s[np++] = b;
+    while (np-- > 0) any_pass<COLS, true, false>(pass_bits(logn, b0s[np]), sm, logn, loglpb, b0s[np], tw);
+}
+
+constexpr int FT = 256;                     // threads of the transform kernels
+
+// the noise of the torus (COARSE: half the 2x2 sums of the torus of twice the
+// sides, so that it stays standard normal: Appendix A, Eq. averaging) and its row
+// transforms, frequencies bit-reversed; 2^loglpb rows a block
+// (first sample = *first_dev + first when first_dev is given: a captured CUDA
+// graph can advance the sample range between replays)
+struct RowArgs {
+    long long lines;
+    int logpx, logpz, loglpb;
+    uint64_t seed;
+    uint32_t level, fld0;
+    int im;                                 // 0: the im lane's field is not wanted
+    int64_t first;
+    const int64_t* first_dev;
+    const NormTab* norm;
+    const cw* tw;
+    fx2* out;
+};
+
+template <bool COARSE>
+__global__ void __launch_bounds__(FT, 3) k_noise_rows(const RowArgs A) {
+    extern __shared__ fx2 sm[];
+    const int logn = A.logpx, n = 1 << logn, lpb = 1 << A.loglpb;
+    const long long line0 = (long long)blockIdx.x << A.loglpb;
+    const int64_t first = (A.first_dev ? *A.first_dev : 0) + A.first;
+    const uint32_t k0 = (uint32_t)A.seed, k1 = (uint32_t)(A.seed >> 32) ^ A.level;
+    auto draw = [&](uint32_t q, int fld, uint64_t sample, long long& y0, long long& y1) {
+        uint32_t c[4] = {q, A.fld0 + (uint32_t)fld, (uint32_t)sample, (uint32_t)(sample >> 32)};
+        philox10(c, k0, k1);
+        normal_pair(c[0], c[1], c[2], c[3], A.norm, y0, y1);
+    };
+    const int lw = COARSE ? logn : logn - 1;          // a thread's unit: a point; two neighbours
+    for (int it = threadIdx.x; it < lpb << lw; it += FT) {
+        const int l = it >> lw, x = it & ((1 << lw) - 1);
+        const long long line = line0 + l;
+        if (line >= A.lines) break;
+        const uint64_t sample = (uint64_t)(first + (line >> A.logpz));
+        const uint32_t row = (uint32_t)(line & ((1ll << A.logpz) - 1));
+        long long y[2][2] = {};
+#pragma unroll 1
+        for (int f = 0; f < (A.im ? 2 : 1); ++f) {
+            long long a, b;
+            if (COARSE) {
+                long long c, d;
+                draw(((2 * row) << logn) + x, f, sample, a, b);
+                draw(((2 * row + 1) << logn) + x, f, sample, c, d);
+                a = (a + b + c + d + 1) >> 1;
+            } else {
+                draw((row << lw) + x, f, sample, a, b);
+            }
+            if (f) { y[1][0] = a; y[1][1] = b; } else { y[0][0] = a; y[0][1] = b; }
+        }
+        if (COARSE) {
+            sm[at<false>(l, x, logn, 0)] = fx2{y[0][0], y[1][0]};
+        } else {
+            sm[at<false>(l, 2 * x, logn, 0)] = fx2{y[0][0], y[1][0]};
+            sm[at<false>(l, 2 * x + 1, logn, 0)] = fx2{y[0][1], y[1][1]};
+        }
+    }
+    __syncthreads();
+    for (int b = 0; b < logn;) {
+        const int w = pass_bits(logn, b);
+        any_pass<false, false, false>(w, sm, logn, A.loglpb, b, A.tw);
+        b += w;
+    }
+    for (int t = threadIdx.x; t < n << A.loglpb; t += FT) {
+        const int l = t >> logn, p = t & (n - 1);
+        if (line0 + l < A.lines) A.out[((line0 + l) << logn) + p] = sm[at<false>(l, p, logn, 0)];
+    }
+}
+
+// column transforms, filter and inverse column transforms of 2^loglpb columns a
+// block, in place; only the window's rows (the first nz) are written
+__global__ void __launch_bounds__(FT, 3)
+k_columns(int logpx, int logpz, int loglpb, int nz, const cw* __restrict__ tw, const wq* __restrict__ filt, fx2* data) {
+    extern __shared__ fx2 sm[];
+    const int c0 = (blockIdx.x & ((1 << (logpx - loglpb)) - 1)) << loglpb, lpb = 1 << loglpb;
+    fx2* d = data + ((size_t)(blockIdx.x >> (logpx - loglpb)) << (logpx + logpz)) + c0;
+    for (int t = threadIdx.x; t < lpb << logpz; t += FT)
+        sm[t] = d[((size_t)(t >> loglpb) << logpx) + (t & (lpb - 1))];
+    __syncthreads();
+    int b = 0, w = pass_bits(logpz, 0);
+    for (; b + w < logpz; w = pass_bits(logpz, b)) {
+        any_pass<true, false, false>(w, sm, logpz, loglpb, b, tw);
+        b += w;
+    }
+    any_pass<true, false, true>(w, sm, logpz, loglpb, b, tw, filt + c0, 1 << logpx);
+    inverse_passes<true>(sm, logpz, loglpb, b, tw);
+    for (int t = threadIdx.x; t < nz << loglpb; t += FT)
+        d[((size_t)(t >> loglpb) << logpx) + (t & (lpb - 1))] = sm[t];
+}
+
+// inverse row transforms of the window's rows (their columns brought to one
+// scale first) -> the pair's two fields, compact [S][nz][nx] real arrays (al
+// may be null: the im lane is unused); nx and nz are powers of two
+__global__ void __launch_bounds__(FT, 3)
+k_rows_window(long long lines, int logpx, int logpz, int loglpb, int lognx, int lognz, const cw* __restrict__ tw,
+              const int* __restrict__ colsh, double scale, const fx2* __restrict__ data, double inv_sigma, PackTr tr,
+              double* lk, double* al) {
+    extern __shared__ fx2 sm[];
+    const int n = 1 << logpx;
+    const long long line0 = (long long)blockIdx.x << loglpb;
+    for (int t = threadIdx.x; t < n << loglpb; t += FT) {
+        const int l = t >> logpx, p = t & (n - 1);
+        const long long line = line0 + l;
+        fx2 v{0, 0};
+        const int sh = colsh[p];
+        if (line < lines && sh < 62) {
+            v = data[((line >> lognz) << (logpx + logpz)) + ((line & ((1ll << lognz) - 1)) << logpx) + p];
+            v = fx2{rshift(v.re, sh), rshift(v.im, sh)};
+        }
+        sm[at<false>(l, p, logpx, 0)] = v;
+    }
+    __syncthreads();
+    inverse_passes<false>(sm, logpx, loglpb, logpx, tw);
+    for (int t = threadIdx.x; t < 1 << (lognx + loglpb); t += FT) {
+        const int l = t >> lognx, i = t & ((1 << lognx) - 1);
+        if (line0 + l >= lines) break;
+        const long long g = ((line0 + l) << lognx) + i;
+        const fx2 v = sm[at<false>(l, i, logpx, 0)];
+        const double re = (double)v.re * scale;
+        lk[g] = tr.re_uniform ? uniform_of(re, inv_sigma, tr.re_a, tr.re_b) : re + tr.re_a;
+        if (al) al[g] = uniform_of((double)v.im * scale, inv_sigma, tr.im_lo, tr.im_span);
+    }
 }
 
 // one 2x2 averaging step of both fields
@@ -224,36 +379,35 @@ inline bool pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
 template <int L>
 int fft_pass(cplx* d, int S, int n, int lines, long long sstride, int lstride, int estride,
-             const cplx* tw, int inverse, cudaStream_t st) {
+             const cplx* tw, cudaStream_t st) {
     size_t sm = (size_t)L * n * sizeof(cplx);
     RICH_CUDA(cudaFuncSetAttribute(k_fft_lines<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     rich_count_launch();
-    k_fft_lines<L><<<(unsigned)S * (lines / L), 256, sm, st>>>(d, n, ilog2(n), lines, sstride, lstride,
-                                                               estride, tw, inverse);
+    k_fft_lines<L><<<(unsigned)S * (lines / L), 256, sm, st>>>(d, n, ilog2(n), lines, sstride, lstride, estride,
+                                                               tw);
     return 0;
 }
 
 // lines per block: the largest of 8, 4, 2, 1 that divides the line count and
 // keeps the block's lines within 128 KB of shared memory
 int fft_dispatch(cplx* d, int S, int n, int lines, long long sstride, int lstride, int estride,
-                 const cplx* tw, int inverse, cudaStream_t st) {
+                 const cplx* tw, cudaStream_t st) {
     for (int L = 8; L >= 1; L >>= 1) {
         if (lines % L || (size_t)L * n * sizeof(cplx) > (128u << 10)) continue;
         switch (L) {
-            case 8: return fft_pass<8>(d, S, n, lines, sstride, lstride, estride, tw, inverse, st);
-            case 4: return fft_pass<4>(d, S, n, lines, sstride, lstride, estride, tw, inverse, st);
-            case 2: return fft_pass<2>(d, S, n, lines, sstride, lstride, estride, tw, inverse, st);
-            default: return fft_pass<1>(d, S, n, lines, sstride, lstride, estride, tw, inverse, st);
+            case 8: return fft_pass<8>(d, S, n, lines, sstride, lstride, estride, tw, st);
+            case 4: return fft_pass<4>(d, S, n, lines, sstride, lstride, estride, tw, st);
+            case 2: return fft_pass<2>(d, S, n, lines, sstride, lstride, estride, tw, st);
+            default: return fft_pass<1>(d, S, n, lines, sstride, lstride, estride, tw, st);
         }
     }
     return RICH_ERR_INVALID;
 }
 
-int fft2(cplx* d, int S, int px, int pz, const cplx* twx, const cplx* twz, int inverse,
-         cudaStream_t st) {
+int fft2(cplx* d, int S, int px, int pz, const cplx* twx, const cplx* twz, cudaStream_t st) {
     const long long ss = (long long)px * pz;
-    if (int e = fft_dispatch(d, S, px, pz, ss, px, 1, twx, inverse, st)) return e;   // rows (x)
-    if (int e = fft_dispatch(d, S, pz, px, ss, 1, px, twz, inverse, st)) return e;   // columns (z)
+    if (int e = fft_dispatch(d, S, px, pz, ss, px, 1, twx, st)) return e;   // rows (x)
+    if (int e = fft_dispatch(d, S, pz, px, ss, 1, px, twz, st)) return e;   // columns (z)
     RICH_CUDA(cudaGetLastError());
     return 0;
 }
@@ -268,7 +422,29 @@ bool bad_field(const rich_field_t* fd) {
            !(fd->nu <= 16);
 }
 
-// sqrt(F c) on a px x pz torus of spacing h, cached in the context
+// exp(-2 pi i k / n), k < n: a quarter turn from the host's functions, the rest
+// by symmetry
+static void make_twiddles(int n, cw* w) {
+    for (int k = 0; k < n; ++k) {
+        if (n < 4 || k < n / 4) {
+            w[k] = circle_point(-k, n);
+        } else {
+            const cw v = w[k - n / 4];
+            w[k] = cw{v.im, neg(v.re)};                       // times -i
+        }
+    }
+}
+
+static const NormTab& norm_tab() {
+    static const NormTab t = [] { NormTab v; make_norm_tab(v); return v; }();
+    return t;
+}
+
+// The filter sqrt(F c) on a px x pz torus of spacing h, with what the transforms
+// read, cached in the context.  Scales: column kx of the filter is in units of
+// 2^e, the power of two above its Euclidean norm (so that its unnormalised
+// inverse transform of unit values stays one); the rows' transforms take the
+// power above the whole filter's norm.
 static int spectrum_on(rich_ctx* ctx, int px, int pz, double h, const rich_field_t* fd,
                        cudaStream_t st, const rich_spectrum** out, double* min_ratio) {
     const double sigma2 = fd->sigma2, corr_len = fd->corr_len, nu = fd->nu;
@@ -284,26 +460,63 @@ static int spectrum_on(rich_ctx* ctx, int px, int pz, double h, const rich_field
     rich_spectrum e{};
     e.px = px; e.pz = pz; e.h = h; e.sigma2 = sigma2; e.corr_len = corr_len; e.corr_len_z = lz; e.nu = nu;
     const CovModel cm{sigma2, corr_len, lz, nu, nu > 0 ? sigma2 * pow(2.0, 1.0 - nu) / tgamma(nu) : 0.0};
-    cplx* c = nullptr;
-    RICH_CUDA(cudaMalloc(&c, sizeof(cplx) * npts));
-    RICH_CUDA(cudaMalloc(&e.tw, sizeof(cplx) * (px / 2 + pz / 2 + 2)));
-    cplx* tw = (cplx*)e.tw;
+    struct Bufs { void *a = nullptr, *b = nullptr, *t = nullptr; ~Bufs() { cudaFree(a); cudaFree(b); cudaFree(t); } } tmp;
+    RICH_CUDA(cudaMalloc(&tmp.a, sizeof(cplx) * npts));
+    RICH_CUDA(cudaMalloc(&tmp.b, sizeof(cplx) * (px / 2 + pz / 2 + 2)));
+    cplx *c = (cplx*)tmp.a, *tw = (cplx*)tmp.b;
     rich_count_launch(); k_twiddles<<<nb(px / 2), 256, 0, st>>>(px, tw);
     rich_count_launch(); k_twiddles<<<nb(pz / 2), 256, 0, st>>>(pz, tw + px / 2 + 1);
     rich_count_launch(); k_cov<<<nb(npts), 256, 0, st>>>(px, pz, h, cm, c);
-    if (int r = fft2(c, 1, px, pz, tw, tw + px / 2 + 1, 0, st)) { cudaFree(c); return r; }
+    if (int r = fft2(c, 1, px, pz, tw, tw + px / 2 + 1, st)) return r;
     std::vector<cplx> hl(npts);
     RICH_CUDA(cudaMemcpyAsync(hl.data(), c, sizeof(cplx) * npts, cudaMemcpyDeviceToHost, st));
     RICH_CUDA(cudaStreamSynchronize(st));
-    double lmin = hl[0].re, lmax = hl[0].re;
-    for (auto& v : hl) { lmin = std::min(lmin, v.re); lmax = std::max(lmax, v.re); }
+    double lmin = hl[0].re, lmax = hl[0].re, sum = 0.0, total = 0.0;
+    std::vector<double> col(px, 0.0);
+    for (int g = 0; g < npts; ++g) {
+        const double v = hl[g].re;
+        lmin = std::min(lmin, v); lmax = std::max(lmax, v);
+        sum += v;
+        if (v > 0.0) { col[g & (px - 1)] += v; total += v; }
+    }
     e.min_ratio = lmin / lmax;
-    RICH_CUDA(cudaMalloc(&e.sq, sizeof(double) * npts));
-    rich_count_launch(); k_sqrt_spec<<<nb(npts), 256, 0, st>>>(npts, c, e.sq);
+    // tables: Q62 twiddles of rows and columns, the normals', the columns'
+    // exponents (natural order) and their distance to the rows' (bit-reversed)
+    const size_t n_tw = sizeof(cw) * (px + pz), o_norm = n_tw, o_e = o_norm + sizeof(NormTab),
+                 o_sh = o_e + sizeof(int) * px, o_f = (o_sh + sizeof(int) * px + 255) & ~(size_t)255;
+    std::vector<char> hb(o_f);
+    cw* htw = (cw*)hb.data();
+    make_twiddles(px, htw);
+    if (pz == px) std::copy(htw, htw + px, htw + px);
+    else make_twiddles(pz, htw + px);
+    *(NormTab*)(hb.data() + o_norm) = norm_tab();
+    const bool finite = std::isfinite(sum);               // (an infinite variance: the fields are NaN)
+    int etot = 0;
+    if (finite) frexp(sqrt(total), &etot);
+    int* he = (int*)(hb.data() + o_e);
+    int* hsh = (int*)(hb.data() + o_sh);
+    const int lx = ilog2(px), lzz = ilog2(pz);
+    for (int k = 0; k < px; ++k) {
+        he[k] = etot - 62;
+        if (finite && col[k] > 0.0) frexp(sqrt(col[k]), &he[k]);
+        he[k] = std::max(he[k], etot - 62);               // below: nothing of it is left in a row
+    }
+    for (int p = 0; p < px; ++p) {
+        int k = 0;
+        for (int b = 0; b < lx; ++b) k |= ((p >> b) & 1) << (lx - 1 - b);
+        hsh[p] = std::max(0, etot - he[k]);
+    }
+    e.scale = finite ? ldexp(1.0, etot - FX_BITS + lx / 2 + lzz / 2 - lx - lzz) : NAN;
+    RICH_CUDA(cudaMalloc(&tmp.t, o_f + sizeof(wq) * (size_t)npts));
+    char* d = (char*)tmp.t;
+    RICH_CUDA(cudaMemcpyAsync(d, hb.data(), o_f, cudaMemcpyHostToDevice, st));
+    e.twx = d; e.twz = (cw*)d + px; e.norm = d + o_norm; e.colsh = (int*)(d + o_sh); e.filt = d + o_f;
+    rich_count_launch(); k_filter_table<<<nb(npts), 256, 0, st>>>(lx, lzz, c, (int*)(d + o_e), (wq*)e.filt);
+    RICH_CUDA(cudaGetLastError());
     RICH_CUDA(cudaStreamSynchronize(st));
-    cudaFree(c);
+    e.tab = tmp.t; tmp.t = nullptr;
     if (ctx->spectra.size() >= 16) {               // bounded cache: drop the oldest
-        cudaFree(ctx->spectra.front().sq); cudaFree(ctx->spectra.front().tw);
+        cudaFree(ctx->spectra.front().tab);
         ctx->spectra.erase(ctx->spectra.begin());
     }
     ctx->spectra.push_back(e);
@@ -340,15 +553,59 @@ static int ensure_work(rich_ctx* ctx, size_t bytes) {
     return 0;
 }
 
-// FFT-MA of the packed noise in `work` ([cs][pz][px] complex) in place
-static int fftma_inplace(cplx* work, int cs, const rich_spectrum* sp, cudaStream_t st) {
-    const int px = sp->px, pz = sp->pz, npts = px * pz;
-    const cplx* twx = (const cplx*)sp->tw;
-    const cplx* twz = twx + px / 2 + 1;
-    if (int e = fft2(work, cs, px, pz, twx, twz, 0, st)) return e;
+// log2 of the lines of n points a block takes: 2048 points (8 a thread, 36 KB of
+// shared memory), fewer while that leaves SMs without a block; at least `least`
+// where 128 KB hold them, and no more than `most`
+static int log_lines(const rich_ctx* ctx, int logn, long long lines, int least, int most) {
+    int l = std::max(11 - logn, least);
+    while (l > 0 && (16ll << (logn + l)) > (64 << 10)) --l;
+    while (l > least && logn + l > 8 && (lines >> l) < ctx->sm_count) --l;
+    return std::min(l, most);
+}
+
+static size_t row_smem(int logn, int loglpb) {
+    return sizeof(fx2) * ((size_t)((1 << logn) + ((1 << logn) >> 3)) << loglpb);
+}
+
+template <typename K>
+static int allow_smem(K kernel, size_t bytes) {
+    if (bytes > (48u << 10))
+        RICH_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return 0;
+}
+
+// FFT-MA of one packed pair of fields for cs samples in `work` ([cs][pz][px]):
+// the window's nx x nz cells to re and im (im null: that lane is not wanted).
+// coarse: the noise is that of the torus of twice the sides, upscaled.
+static int fftma(rich_ctx* ctx, const rich_spectrum* sp, fx2* work, int cs, uint64_t seed, uint32_t level,
+                 int64_t first, const int64_t* first_dev, uint32_t fld0, bool coarse, int nx, int nz,
+                 double inv_sigma, const PackTr& tr, double* re, double* im, cudaStream_t st) {
+    const int lx = ilog2(sp->px), lz = ilog2(sp->pz), lnx = ilog2(nx), lnz = ilog2(nz);
+    RowArgs A{};
+    A.lines = (long long)cs << lz;
+    A.logpx = lx; A.logpz = lz; A.loglpb = log_lines(ctx, lx, A.lines, 0, 11);
+    A.seed = seed; A.level = level; A.fld0 = fld0; A.im = im != nullptr; A.first = first; A.first_dev = first_dev;
+    A.norm = (const NormTab*)sp->norm; A.tw = (const cw*)sp->twx; A.out = work;
+    size_t smem = row_smem(lx, A.loglpb);
+    auto* rows = coarse ? k_noise_rows<true> : k_noise_rows<false>;
+    if (int e = allow_smem(rows, smem)) return e;
     rich_count_launch();
-    k_filter<<<nb((long long)cs * npts), 256, 0, st>>>(cs, npts, sp->sq, work);
-    if (int e = fft2(work, cs, px, pz, twx, twz, 1, st)) return e;
+    rows<<<(unsigned)((A.lines + (1ll << A.loglpb) - 1) >> A.loglpb), FT, smem, st>>>(A);
+    // columns: eight side by side fill a 128-byte line
+    const int lc = log_lines(ctx, lz, (long long)cs << lx, std::min(3, lx), lx);
+    smem = sizeof(fx2) << (lz + lc);
+    if (int e = allow_smem(k_columns, smem)) return e;
+    rich_count_launch();
+    k_columns<<<(unsigned)((long long)cs << (lx - lc)), FT, smem, st>>>(lx, lz, lc, nz, (const cw*)sp->twz,
+                                                                       (const wq*)sp->filt, work);
+    const long long wl = (long long)cs << lnz;
+    const int lw = log_lines(ctx, lx, wl, 0, 11);
+    smem = row_smem(lx, lw);
+    if (int e = allow_smem(k_rows_window, smem)) return e;
+    rich_count_launch();
+    k_rows_window<<<(unsigned)((wl + (1ll << lw) - 1) >> lw), FT, smem, st>>>(
+        wl, lx, lz, lw, lnx, lnz, (const cw*)sp->twx, sp->colsh, sp->scale, work, inv_sigma, tr, re, im);
+    RICH_CUDA(cudaGetLastError());
     return 0;
 }
 
@@ -377,10 +634,10 @@ static int packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int nz, u
     const rich_spectrum* sp = nullptr;
     if (int e = spectrum_on(ctx, px, pz, 1.0 / nz, fd, st, &sp, nullptr)) return e;
     const int npts = px * pz;
-    const size_t per = (size_t)npts * sizeof(cplx) + 32 * (size_t)nx * nz;
+    const size_t per = (size_t)npts * sizeof(fx2) + (coarsen ? 32 * (size_t)nx * nz : 0);
     const int chunk = (int)std::max<size_t>(1, CHUNK_BYTES / per);
     if (int e = ensure_work(ctx, per * std::min(chunk, S))) return e;
-    cplx* work = (cplx*)ctx->field_work;
+    fx2* work = (fx2*)ctx->field_work;
     const int cap = std::min(chunk, S);
     double* tmp = (double*)(work + (size_t)npts * cap);   // [cap][4][nz][nx] real scratch
     const int nxo = nx >> coarsen, nzo = nz >> coarsen;
@@ -389,10 +646,6 @@ static int packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int nz, u
         int cs = std::min(cap, S - s0);
         for (int k = 0; k < npk; ++k) {
             const Pack& P = pk[k];
-            rich_count_launch();
-            k_noise<<<nb((long long)cs * (npts / 2)), 256, 0, st>>>(cs, npts, fd->seed, level, first + s0,
-                                                                     first_dev, work, P.fld0);
-            if (int e = fftma_inplace(work, cs, sp, st)) return e;
             // real scratch: two ping-pong pairs of [cs][nz][nx] arrays
             const size_t blk = (size_t)cs * nx * nz;
             double* bl[2] = {tmp, tmp + 2 * blk};
@@ -400,9 +653,9 @@ static int packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int nz, u
             const bool im = P.out_im != nullptr;
             double* wl = coarsen ? bl[0] : P.out_re + (size_t)s0 * nx * nz;
             double* wa = !im ? nullptr : coarsen ? ba[0] : P.out_im + (size_t)s0 * nx * nz;
-            rich_count_launch();
-            k_window<<<nb((long long)cs * nx * nz), 256, 0, st>>>(cs, nx, nz, px, pz, work, inv_sigma, P.tr,
-                                                                wl, wa);
+            if (int e = fftma(ctx, sp, work, cs, fd->seed, level, first + s0, first_dev, P.fld0, false, nx, nz,
+                              inv_sigma, P.tr, wl, wa, st))
+                return e;
             int cx = nx, cz = nz, cur = 0;
             for (int c = 0; c < coarsen; ++c) {
                 int ncx = cx / 2, ncz = cz / 2;
@@ -449,21 +702,6 @@ int rich_soil_device(rich_ctx* ctx, const rich_field_t* fd, const rich_soil_mode
     return packs_device(ctx, fd, nx, nz, level, first, S, coarsen, npk, pk, st, nullptr);
 }
 
-namespace {
-// coarse white noise by 2x2 averaging on the torus, scaled by 1/2 so that it
-// stays standard normal (Appendix A, Eq. averaging); both packed fields at once
-__global__ void k_noise_upscale(int S, int pxc, int pzc, const cplx* __restrict__ y, cplx* yc) {
-    long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int nc = pxc * pzc, fx = 2 * pxc;
-    if (g >= (long long)S * nc) return;
-    int s = (int)(g / nc), q = (int)(g - (long long)s * nc);
-    int J = q / pxc, I = q - J * pxc;
-    const cplx* b = y + (size_t)s * 4 * nc + (size_t)(2 * J) * fx + 2 * I;
-    cplx a = b[0], c = b[1], d = b[fx], e = b[fx + 1];
-    yc[g] = cplx{0.5 * (a.re + c.re + d.re + e.re), 0.5 * (a.im + c.im + d.im + e.im)};
-}
-}
-
 // one packed pair of fields drawn as a fine/coarse couple: outputs on the
 // fine grid (f_*) and on the half grid (c_*); im outputs null: lane unused
 struct PairPack {
@@ -489,33 +727,24 @@ static int pair_packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int 
     // spectrum_on may reallocate the cache vector: look both up again
     spectrum_on(ctx, px, pz, 1.0 / nz, fd, st, &spf, nullptr);
     spectrum_on(ctx, px / 2, pz / 2, 2.0 / nz, fd, st, &spc, nullptr);
-    const int npf = px * pz, npc = npf / 4;
-    const size_t per = (size_t)(npf + npc) * sizeof(cplx);
+    const int npf = px * pz;
+    const size_t per = (size_t)npf * sizeof(fx2);
     const int cap = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, CHUNK_BYTES / per));
     if (int e = ensure_work(ctx, per * cap)) return e;
-    cplx* wf = (cplx*)ctx->field_work;
-    cplx* wc = wf + (size_t)npf * cap;
+    fx2* work = (fx2*)ctx->field_work;         // the two members take turns
     const double inv_sigma = 1.0 / sqrt(fd->sigma2);
     const int ncx = nx / 2, ncz = nz / 2;
     for (int s0 = 0; s0 < S; s0 += cap) {
         int cs = std::min(cap, S - s0);
         for (int k = 0; k < npk; ++k) {
             const PairPack& P = pk[k];
-            rich_count_launch();
-            k_noise<<<nb((long long)cs * (npf / 2)), 256, 0, st>>>(cs, npf, fd->seed, level, first + s0, nullptr,
-                                                                    wf, P.fld0);
-            rich_count_launch();
-            k_noise_upscale<<<nb((long long)cs * npc), 256, 0, st>>>(cs, px / 2, pz / 2, wf, wc);
-            if (int e = fftma_inplace(wf, cs, spf, st)) return e;
-            if (int e = fftma_inplace(wc, cs, spc, st)) return e;
-            rich_count_launch();
-            k_window<<<nb((long long)cs * nx * nz), 256, 0, st>>>(
-                cs, nx, nz, px, pz, wf, inv_sigma, P.tr, P.f_re + (size_t)s0 * nx * nz,
-                P.f_im ? P.f_im + (size_t)s0 * nx * nz : nullptr);
-            rich_count_launch();
-            k_window<<<nb((long long)cs * ncx * ncz), 256, 0, st>>>(
-                cs, ncx, ncz, px / 2, pz / 2, wc, inv_sigma, P.tr, P.c_re + (size_t)s0 * ncx * ncz,
-                P.c_im ? P.c_im + (size_t)s0 * ncx * ncz : nullptr);
+            const size_t of = (size_t)s0 * nx * nz, oc = (size_t)s0 * ncx * ncz;
+            if (int e = fftma(ctx, spf, work, cs, fd->seed, level, first + s0, nullptr, P.fld0, false, nx, nz,
+                              inv_sigma, P.tr, P.f_re + of, P.f_im ? P.f_im + of : nullptr, st))
+                return e;
+            if (int e = fftma(ctx, spc, work, cs, fd->seed, level, first + s0, nullptr, P.fld0, true, ncx, ncz,
+                              inv_sigma, P.tr, P.c_re + oc, P.c_im ? P.c_im + oc : nullptr, st))
+                return e;
         }
     }
     RICH_CUDA(cudaGetLastError());

@@ -39,12 +39,15 @@ struct rich_samplebuf {
     int last_occ = 1;                           // resident CTAs per SM of the last fused launch
 };
 
-// sqrt of the circulant covariance spectrum on one torus (+ FFT twiddles)
+// filter (square root of the circulant covariance spectrum) on one torus and
+// the fixed-point tables of its transforms (fields.cu), in one allocation
 struct rich_spectrum {
     int px = 0, pz = 0;
     double h = 0, sigma2 = 0, corr_len = 0, corr_len_z = 0, nu = 0, min_ratio = 0;
-    double* sq = nullptr;                       // [pz][px]
-    void* tw = nullptr;                         // twiddles of both line lengths
+    void* tab = nullptr;                        // the allocation
+    const void *twx = nullptr, *twz = nullptr, *norm = nullptr, *filt = nullptr;
+    const int* colsh = nullptr;                 // per column, bit-reversed: shift to the rows' scale
+    double scale = 0;                           // a unit of the result
 };
 
 // Live timing of the finest-level smoothing launches (the dominant kernel):
