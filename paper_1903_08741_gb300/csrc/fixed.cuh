@@ -1,5 +1,5 @@
-// 64-bit fixed-point arithmetic of the field generator: complex products, FFT
-// butterflies and standard normals in integers.
+// 64-bit fixed-point arithmetic: the field generator's complex products, FFT
+// butterflies and standard normals, and the closures' elementary functions.
 //
 // Why integers: GB300 issues 2 FP64 operations per SM and clock, a radix-2 FP64
 // butterfly with its twiddle takes 8 of them (4 clocks a lane), and the normals
@@ -14,6 +14,7 @@
 #pragma once
 #include <stdint.h>
 #include <math.h>
+#include <string.h>
 
 namespace rich_fx {
 
@@ -221,6 +222,128 @@ FX void normal_pair(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const No
     const int sh = 62 - FX_BITS - t;                  // at least 3: |y| < 2^4
     y0 = sh > 62 ? 0 : rshift(rmul(cb, qs), sh);
     y1 = sh > 62 ? 0 : rshift(rmul(sb, qs), sh);
+}
+
+// ---------------------------------------------------------------- exp and log
+// The closures' elementary functions without the FP64 pipe (CUDA's exp holds it
+// for 16 multiply-adds, this one for none and about 70 integer instructions on
+// pipes 16 times as wide).  Tables and remainders after Tang (ACM TOMS 15, 1989
+// and 16, 1990); working precision 2^-60.
+#ifdef __CUDACC__
+#define FX_TABLE static __device__ const
+#else
+#define FX_TABLE static const
+#endif
+#include "fixed_tables.cuh"
+
+constexpr unsigned long long LN2_128 = 0x58B90BFBE8E7BCull;  // ln 2 / 128: Q62 and the next 32 bits
+constexpr unsigned int LN2_128_LO = 0xD5E4F1D9u;
+
+// 2^(k/128) e^r = v 2^n: v in Q62, 1 <= v < 2 (up to rounding); r in Q62, |r| < 2^-7.9
+FX unsigned long long exp_core(int k, long long r, int& n) {
+    const int r31 = (int)(r >> 31);
+    const int c24 = (int)((1ll << 31) / 24) + (int)(wide(r31, (int)((1ll << 31) / 120)) >> 31);
+    long long p = (1ll << 62) / 6 + wide(r31, c24);
+    p = (1ll << 61) + rmul(r, p);
+    p = r + rmul(rmul(r, r), p);
+    const long long t = EXP_TAB[k & 127];
+    n = k >> 7;
+    const unsigned long long v = (unsigned long long)(t + rmul(t, p));
+    if (v >> 62) return v;
+    --n;                                                     // 2^0 e^r with r < 0
+    return v << 1;
+}
+
+// v 2^n (v in Q62) rounded to FP64; the result is normal
+FX double fx_to_double(unsigned long long v, int n) {
+    const unsigned long long m = (v + 512) >> 10;            // 2^52 <= m <= 2^53
+    const unsigned long long b = m + ((unsigned long long)(n + 1022) << 52);
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double d; memcpy(&d, &b, 8); return d;
+#endif
+}
+FX unsigned long long double_bits(double x) {
+#ifdef __CUDA_ARCH__
+    return (unsigned long long)__double_as_longlong(x);
+#else
+    unsigned long long b; memcpy(&b, &x, 8); return b;
+#endif
+}
+
+// exp(x) to 0.54 units in the last place for |x| < 512 (any other x: the library's)
+FX double fx_exp(double x) {
+    const unsigned long long b = double_bits(x);
+    const int e = (int)(b >> 52 & 0x7FF) - 1023;
+    if (e >= 9 || e < -60) return exp(x);                    // large, NaN; tiny, zero
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    int k = 0;
+    if (e >= -8) {                                           // round(|x| 128 / ln 2)
+        const unsigned long long q = (m >> 21) * 0xB8AA3B29ull;
+        k = (int)((q + (1ull << (54 - e))) >> (55 - e));
+    }
+    long long r = e >= -10 ? (long long)(m << (e + 10)) : (long long)(m >> -(e + 10));   // |x| in Q62 mod 4
+    r -= (long long)((unsigned long long)k * LN2_128 + (((unsigned long long)k * LN2_128_LO) >> 32));
+    if (b >> 63) { k = -k; r = -r; }
+    int n;
+    const unsigned long long v = exp_core(k, r, n);
+    return fx_to_double(v, n);
+}
+
+// e^(y 2^-F), |y 2^-F| < 512, as v 2^n
+template <int F>
+FX unsigned long long exp_fixed(long long y, int& n) {
+    const int k = (int)((wide((int)(y >> (F - 22)), 1549082005) + (1ll << 44)) >> 45);     // 128 / ln 2 in Q23
+    const unsigned long long c = (unsigned long long)(long long)k * LN2_128 +
+                                 (unsigned long long)(((long long)k * (long long)LN2_128_LO) >> 32);
+    return exp_core(k, (long long)(((unsigned long long)y << (62 - F)) - c), n);
+}
+template <int F>
+FX double exp_fixed(long long y) {
+    int n;
+    const unsigned long long v = exp_fixed<F>(y, n);
+    return fx_to_double(v, n);
+}
+
+// ln(M 2^(e-59)) in Q57, 2^59 <= M < 2^60, |e| < 90
+FX long long log_fixed(unsigned long long M, int e) {
+    const int i = (int)(M >> 51) & 255;
+    const long long r = (long long)(M * (unsigned long long)LOG_INV[i]) >> 1;
+    return e * LN2_57 + LOG_TAB[i] + ((log1p70(r) + 4096) >> 13);
+}
+
+// van Genuchten saturation at -p = ap/a, in logarithms: with L = ln ap,
+// s = (1 + ap^n)^-m = e^t.  False where a value leaves the fixed-point ranges
+// (2^-59 <= ap < 2^59, 2^-6 <= n < 16, 2^-20 <= m < 1, 2^-369 < ap^n < 2^58).
+struct VgLog { long long t, g, l1; };       // t in Q57; g = (n - 1) L in Q53; l1 = ln(1 + ap^n) in Q57
+FX bool vg_log(double ap, double n, double m, VgLog& o) {
+    const unsigned long long ba = double_bits(ap), bn = double_bits(n), bm = double_bits(m), one = 1ull << 52;
+    const int ea = (int)(ba >> 52) - 1023, en = (int)(bn >> 52) - 1023, em = (int)(bm >> 52) - 1023;   // (negative: > 1024)
+    if (ea < -59 || ea > 58 || en < -6 || en > 3 || em < -20 || em > -1) return false;
+    const long long L = log_fixed(((ba & (one - 1)) | one) << 7, ea);
+    const long long y = rmul(L, (long long)(((bn & (one - 1)) | one) << (en + 6)));          // n L in Q53
+    if (y >= 256ll << 53 || y <= -(256ll << 53)) return false;
+    int ne;
+    const unsigned long long v = exp_fixed<53>(y, ne);                                       // ap^n
+    if (ne > 57) return false;
+    const unsigned long long W = ne >= 0 ? v + (1ull << (62 - ne)) : (1ull << 62) + (ne > -63 ? v >> -ne : 0);
+    const int z = clz64(W);
+    o.l1 = log_fixed((W << z) >> 4, (ne > 0 ? ne : 0) + 1 - z);
+    const unsigned long long mm = (bm & (one - 1)) | one;
+    o.t = -rmul(o.l1, (long long)(em >= -10 ? mm << (em + 10) : mm >> -(em + 10)));
+    o.g = y - (L >> 4);
+    return true;
+}
+// s
+FX double vg_s(const VgLog& o) { return exp_fixed<57>(o.t); }
+// the relative conductivity sqrt(s) (1 - s ap^n / ap)^2 and ds/dp / (m n a) =
+// s ap^n / (ap (1 + ap^n))
+FX void vg_k(const VgLog& o, double& krw, double& d) {
+    const long long q = o.g + (o.t >> 4);
+    const double b = 1.0 - exp_fixed<53>(q);
+    krw = exp_fixed<57>(o.t >> 1) * b * b;
+    d = exp_fixed<53>(q - (o.l1 >> 4));
 }
 
 // the tables, from the host's long double functions

@@ -37,6 +37,7 @@
 
 #pragma once
 #include "rich_internal.cuh"
+#include "fixed.cuh"
 #include <math.h>
 #include <type_traits>
 
@@ -818,13 +819,25 @@ __device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool re
 // m n = n - 1, (an / (1 + an))^m = an^m S = (an / (a|p|)) S: one exp fewer
 // than exp(m (n log(a|p|) - log1p(an))), and no cancellation between the two
 // logarithms in the dry limit.
+// The fixed-point evaluation (fixed.cuh) takes every soil of practice; what
+// leaves its ranges takes the FP64 functions.
 __device__ __forceinline__ double vg_sat(double a, double n, double m, double p) {
-    return exp(-m * log1p(exp(n * log(-a * p))));
+    const double ap = -a * p;
+    rich_fx::VgLog o;
+    if (rich_fx::vg_log(ap, n, m, o)) return rich_fx::vg_s(o);
+    return exp(-m * log1p(exp(n * log(ap))));
 }
 
 __device__ __forceinline__ void vg_eval(double a, double n, double m, double p, double& S, double& krw,
                                         double& dS) {
     const double ap = -a * p;
+    rich_fx::VgLog o;
+    if (rich_fx::vg_log(ap, n, m, o)) {
+        S = rich_fx::vg_s(o);
+        rich_fx::vg_k(o, krw, dS);
+        dS *= m * n * a;
+        return;
+    }
     const double an = exp(n * log(ap));
     const double l1 = log1p(an);
     S = exp(-m * l1);
@@ -927,7 +940,7 @@ struct Cta {
         for (int q = tid; q < nc; q += nt) {
             double pp = p[q];
             if constexpr (CL == 0) {
-                thold[q] = pp < 0.0 ? tr + (ts - tr) * exp(aa[q] * pp) : ts;
+                thold[q] = pp < 0.0 ? tr + (ts - tr) * rich_fx::fx_exp(aa[q] * pp) : ts;
             } else {
                 const double r = trc[q], t = tsc[q];
                 thold[q] = pp < 0.0 ? r + (t - r) * vg_sat(aa[q], nn[q], mm[q], pp) : t;
@@ -954,7 +967,7 @@ struct Cta {
             if constexpr (CL == 0) {
                 if (pp < 0.0) {
                     double a = aa[q];
-                    double E = exp(a * pp);
+                    double E = rich_fx::fx_exp(a * pp);
                     K[q] = ks * E;
                     th[q] = tr + (ts - tr) * E;
                     F.Cdt[q] = ((ts - tr) * a * E) * idt;
