@@ -20,8 +20,10 @@ namespace rich_fx {
 
 #ifdef __CUDACC__
 #define FX __host__ __device__ __forceinline__
+#define FXD __device__ __forceinline__       // reads the tables of device memory
 #else
 #define FX inline
+#define FXD inline
 #endif
 
 constexpr int FX_BITS = 55;                 // a standard normal is 2^55
@@ -240,7 +242,7 @@ constexpr unsigned long long LN2_128 = 0x58B90BFBE8E7BCull;  // ln 2 / 128: Q62 
 constexpr unsigned int LN2_128_LO = 0xD5E4F1D9u;
 
 // 2^(k/128) e^r = v 2^n: v in Q62, 1 <= v < 2 (up to rounding); r in Q62, |r| < 2^-7.9
-FX unsigned long long exp_core(int k, long long r, int& n) {
+FXD unsigned long long exp_core(int k, long long r, int& n) {
     const int r31 = (int)(r >> 31);
     const int c24 = (int)((1ll << 31) / 24) + (int)(wide(r31, (int)((1ll << 31) / 120)) >> 31);
     long long p = (1ll << 62) / 6 + wide(r31, c24);
@@ -273,7 +275,7 @@ FX unsigned long long double_bits(double x) {
 }
 
 // exp(x) to 0.54 units in the last place for |x| < 512 (any other x: the library's)
-FX double fx_exp(double x) {
+FXD double fx_exp(double x) {
     const unsigned long long b = double_bits(x);
     const int e = (int)(b >> 52 & 0x7FF) - 1023;
     if (e >= 9 || e < -60) return exp(x);                    // large, NaN; tiny, zero
@@ -293,21 +295,21 @@ FX double fx_exp(double x) {
 
 // e^(y 2^-F), |y 2^-F| < 512, as v 2^n
 template <int F>
-FX unsigned long long exp_fixed(long long y, int& n) {
+FXD unsigned long long exp_fixed(long long y, int& n) {
     const int k = (int)((wide((int)(y >> (F - 22)), 1549082005) + (1ll << 44)) >> 45);     // 128 / ln 2 in Q23
     const unsigned long long c = (unsigned long long)(long long)k * LN2_128 +
                                  (unsigned long long)(((long long)k * (long long)LN2_128_LO) >> 32);
     return exp_core(k, (long long)(((unsigned long long)y << (62 - F)) - c), n);
 }
 template <int F>
-FX double exp_fixed(long long y) {
+FXD double exp_fixed(long long y) {
     int n;
     const unsigned long long v = exp_fixed<F>(y, n);
     return fx_to_double(v, n);
 }
 
 // ln(M 2^(e-59)) in Q57, 2^59 <= M < 2^60, |e| < 90
-FX long long log_fixed(unsigned long long M, int e) {
+FXD long long log_fixed(unsigned long long M, int e) {
     const int i = (int)(M >> 51) & 255;
     const long long r = (long long)(M * (unsigned long long)LOG_INV[i]) >> 1;
     return e * LN2_57 + LOG_TAB[i] + ((log1p70(r) + 4096) >> 13);
@@ -317,7 +319,7 @@ FX long long log_fixed(unsigned long long M, int e) {
 // s = (1 + ap^n)^-m = e^t.  False where a value leaves the fixed-point ranges
 // (2^-59 <= ap < 2^59, 2^-6 <= n < 16, 2^-20 <= m < 1, 2^-369 < ap^n < 2^58).
 struct VgLog { long long t, g, l1; };       // t in Q57; g = (n - 1) L in Q53; l1 = ln(1 + ap^n) in Q57
-FX bool vg_log(double ap, double n, double m, VgLog& o) {
+FXD bool vg_log(double ap, double n, double m, VgLog& o) {
     const unsigned long long ba = double_bits(ap), bn = double_bits(n), bm = double_bits(m), one = 1ull << 52;
     const int ea = (int)(ba >> 52) - 1023, en = (int)(bn >> 52) - 1023, em = (int)(bm >> 52) - 1023;   // (negative: > 1024)
     if (ea < -59 || ea > 58 || en < -6 || en > 3 || em < -20 || em > -1) return false;
@@ -336,10 +338,10 @@ FX bool vg_log(double ap, double n, double m, VgLog& o) {
     return true;
 }
 // s
-FX double vg_s(const VgLog& o) { return exp_fixed<57>(o.t); }
+FXD double vg_s(const VgLog& o) { return exp_fixed<57>(o.t); }
 // the relative conductivity sqrt(s) (1 - s ap^n / ap)^2 and ds/dp / (m n a) =
 // s ap^n / (ap (1 + ap^n))
-FX void vg_k(const VgLog& o, double& krw, double& d) {
+FXD void vg_k(const VgLog& o, double& krw, double& d) {
     const long long q = o.g + (o.t >> 4);
     const double b = 1.0 - exp_fixed<53>(q);
     krw = exp_fixed<57>(o.t >> 1) * b * b;

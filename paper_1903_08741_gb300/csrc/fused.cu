@@ -25,7 +25,9 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 // depend on where an array lives.
 constexpr int WARP_CELLS = 256;
 
-static void plan_smem(FParams& P, int nt) {
+// A cluster (cells > 0) runs its levels of at least `cells` cells on all its CTAs
+// (lx of them): their corrections, and the next level's, stay in the slot.
+static void plan_smem(FParams& P, int nt, long long cells = 0) {
     const size_t w = P.mixed ? 4 : 8;
     const int c = P.nlev - 1;
     const size_t nnc = (size_t)P.nx[c] * P.nz[c];
@@ -44,6 +46,8 @@ static void plan_smem(FParams& P, int nt) {
     P.lw = P.nlev;
     for (int l = 1; l < P.nlev && nt > 32; ++l)
         if ((size_t)P.nx[l] * P.nz[l] <= (size_t)WARP_CELLS) { P.lw = l; break; }
+    P.lx = 0;
+    while (cells > 0 && P.lx < std::min(P.lw, P.nlev - 1) - 1 && (long long)P.nx[P.lx] * P.nz[P.lx] >= cells) ++P.lx;
     for (int l = P.lw; l < P.nlev; ++l) {
         const size_t nc = (size_t)P.nx[l] * P.nz[l];
         if (!P.mixed) {
@@ -59,7 +63,7 @@ static void plan_smem(FParams& P, int nt) {
             off = al16(off + nc * w);
         }
     }
-    for (int l = P.lw - 1; l >= 0; --l) {
+    for (int l = P.lw - 1; l >= (P.lx > 0 ? P.lx + 1 : 0); --l) {
         const size_t bytes = al16((size_t)P.nx[l] * P.nz[l] * w);
         if (off + bytes > budget) break;
         P.osm[l] = (long long)off;
@@ -144,9 +148,16 @@ static int fused_occupancy(const FParams& P, size_t smem, int nt, int* occ) {
     return P.mixed ? rich_occ_g32(P, smem, nt, occ) : rich_occ_g64(P, smem, nt, occ);
 }
 
-static int fused_launch(const FParams& P, int grid, size_t smem, int nt, cudaStream_t st) {
+static int fused_cluster(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
+    if (P.closure == RICH_VAN_GENUCHTEN)
+        return P.mixed ? rich_cluster_vg32(P, smem, n, clusters, st, fit) : rich_cluster_vg64(P, smem, n, clusters, st, fit);
+    return P.mixed ? rich_cluster_g32(P, smem, n, clusters, st, fit) : rich_cluster_g64(P, smem, n, clusters, st, fit);
+}
+
+static int fused_launch(const FParams& P, int grid, size_t smem, int nt, cudaStream_t st, int cluster = 0) {
     RICH_CUDA(cudaMemsetAsync(P.queue, 0, sizeof(int), st));
     rich_count_launch();
+    if (cluster > 1) return fused_cluster(P, smem, cluster, grid, st, nullptr);
     if (P.closure == RICH_VAN_GENUCHTEN) {
         if (P.mixed) rich_launch_vg32(P, grid, smem, nt, st);
         else rich_launch_vg64(P, grid, smem, nt, st);
@@ -184,6 +195,33 @@ static int default_threads(long long nc, int S, int sms) {
     return nc > 32768 || per_sm <= 2 ? 1024 : 512;
 }
 
+// Smallest level that a cluster runs on all its CTAs, and the smallest grid that
+// takes a cluster.  ms without / with (CTAs a sample), levels from 64^2 or 128^2:
+//   FP64:  64^2 x 1 146 / 104 (8), 64^2 x 48 314 / 265 (3), 128^2 x 24 220 / 102 (6;
+//          110 from 128^2), 128^2 x 76 181 / 118 (2; 121)
+//   mixed: 128^2 x 24 116 / 69 (6; 75 from 64^2), 128^2 x 76 100 / 71 (2; 80),
+//          256^2 x 24 247 / 86 (6; 90)
+// An FP64 half-sweep of a 32^2 level is 1024 clocks of one SM's FP64 pipe, about
+// what the barrier costs; FP32 cells are cheaper, so their line lies higher.
+constexpr long long CLUSTER_CELLS64 = 4096, CLUSTER_CELLS32 = 16384;
+
+// CTAs of a sample's cluster (0: one CTA per sample), with the plan of shared
+// memory made for it.  Only where the launch shape is free (rich_set_tuning 0),
+// for V-cycles, and when clusters for all samples are resident together.
+static int pick_cluster(const rich_ctx* ctx, const rich_problem_t* pb, int S, FParams& P, int* cluster) {
+    *cluster = 0;
+    const long long cells = P.mixed ? CLUSTER_CELLS32 : CLUSTER_CELLS64;
+    if (ctx->tune_threads || P.gamma > 1 || (long long)pb->nx * pb->nz < cells || 2ll * S > ctx->sm_count) return 0;
+    plan_smem(P, 512, cells);
+    if (P.lx == 0) return 0;
+    for (int n = std::min(8, ctx->sm_count / S); n >= 2; --n) {
+        int fit = 0;
+        if (int e = fused_cluster(P, fused_smem(P), n, S, nullptr, &fit)) return e;
+        if (fit >= S) { *cluster = n; return 0; }
+    }
+    return 0;
+}
+
 // Fused persistent solve of S samples; stats arrays live in ctx->ws, the
 // per-CTA slots and the queue counter in ctx->fused_scratch.
 int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const double* lnKs,
@@ -196,7 +234,10 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
                     ctx->tune_threads == 32 || ctx->tune_threads == 512)
                        ? ctx->tune_threads : default_threads((long long)pb->nx * pb->nz, S, ctx->sm_count);
     if (int e = fused_setup(pb, S, P)) return e;
-    plan_smem(P, nt);
+    // a cluster of CTAs per sample where they all fit at once (grid: the clusters)
+    int occ = 1, cluster = 0, grid = S;
+    if (int e = pick_cluster(ctx, pb, S, P, &cluster)) return e;
+    if (cluster == 0) plan_smem(P, nt);
     if (soil) {
         P.n_in = soil->n; P.ts_in = soil->theta_s; P.tr_in = soil->theta_r;
         P.alpha_shift = soil->alpha_shift; P.n_shift = soil->n_shift;
@@ -204,9 +245,10 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     const size_t off = (size_t)P.slot_bytes;
     const size_t smem = fused_smem(P);
     P.mixed_inner = ctx->tune_mixed_inner > 0 ? ctx->tune_mixed_inner : MIXED_INNER_DEFAULT;
-    int occ = 0;
-    if (int e = fused_occupancy(P, smem, nt, &occ)) return e;
-    const int grid = std::max(1, std::min(S, ctx->sm_count * occ));
+    if (cluster == 0) {
+        if (int e = fused_occupancy(P, smem, nt, &occ)) return e;
+        grid = std::max(1, std::min(S, ctx->sm_count * occ));
+    }
     const size_t need = (size_t)grid * off + 256;
     if (ctx->fused_bytes < need) {
         if (ctx->fused_scratch) cudaFree(ctx->fused_scratch);
@@ -224,7 +266,7 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     // resident capacity is spread over the SMs first
     w.last_occ = std::max(1, std::min(occ, (grid + ctx->sm_count - 1) / std::max(ctx->sm_count, 1)));
     rich_prof_begin(ctx, st);
-    if (int e = fused_launch(P, grid, smem, nt, st)) return e;
+    if (int e = fused_launch(P, grid, smem, nt, st, cluster)) return e;
     rich_prof_end(ctx, st, 0.0, 0.0);
     w.last = S;
     if (status)

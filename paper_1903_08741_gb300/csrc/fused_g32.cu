@@ -12,4 +12,8 @@ void rich_launch_g32(const FParams& P, int grid, size_t smem, int nt, cudaStream
     launch_shapes<float, 0>(P, grid, smem, nt, st);
 }
 
+int rich_cluster_g32(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
+    return cluster_call<float, 0>(P, smem, n, clusters, st, fit);
+}
+
 }  // namespace rich_fused

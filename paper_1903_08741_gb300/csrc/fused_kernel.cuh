@@ -38,6 +38,7 @@
 #pragma once
 #include "rich_internal.cuh"
 #include "fixed.cuh"
+#include <cooperative_groups.h>
 #include <math.h>
 #include <type_traits>
 
@@ -66,6 +67,7 @@ struct FParams {
                                             // byte offset (-1: in the slot)
     long long osm_alt;                      // likewise the finest level's second red half
     int lw;                                 // first level run by warp 0 alone (nlev: none)
+    int lx;                                 // a cluster's sample: levels below lx run on all its CTAs
     long long s64[MAXL][N64];               // levels >= lw: every array in dynamic shared
     long long smg[MAXL][NMG];               // memory at these byte offsets (-1: not there)
     long long smem_bytes;                   // dynamic shared memory of a CTA
@@ -135,6 +137,10 @@ void rich_launch_g64(const FParams& P, int grid, size_t smem, int nt, cudaStream
 void rich_launch_g32(const FParams& P, int grid, size_t smem, int nt, cudaStream_t st);
 void rich_launch_vg64(const FParams& P, int grid, size_t smem, int nt, cudaStream_t st);
 void rich_launch_vg32(const FParams& P, int grid, size_t smem, int nt, cudaStream_t st);
+int rich_cluster_g64(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit);
+int rich_cluster_g32(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit);
+int rich_cluster_vg64(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit);
+int rich_cluster_vg32(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit);
 // the adjoint kernel's instantiations (fused_adj64.cu, fused_adj32.cu): the
 // kernel's address (occupancy queries) and its launch with 512 threads
 const void* rich_adjoint_kernel64(bool wcycle);
@@ -270,6 +276,14 @@ struct GWarp {
     static __device__ __forceinline__ int rank() { return threadIdx.x & 31; }
     static __device__ __forceinline__ int size() { return 32; }
     static __device__ __forceinline__ void sync() { __syncwarp(); }
+};
+// all CTAs of a thread-block cluster (one sample): the barrier orders their
+// global and shared accesses
+struct GClu {
+    static __device__ __forceinline__ cooperative_groups::cluster_group c() { return cooperative_groups::this_cluster(); }
+    static __device__ __forceinline__ int rank() { return (int)(c().block_rank() * blockDim.x + threadIdx.x); }
+    static __device__ __forceinline__ int size() { return (int)(c().num_blocks() * blockDim.x); }
+    static __device__ __forceinline__ void sync() { c().sync(); }
 };
 
 // Gauss-Seidel value of a cell (storage indices b) from its current
@@ -728,30 +742,45 @@ __device__ __forceinline__ void gwalk(const Lv<T>* L, int root, int nlev, int lw
 
 // V-cycle with the levels from lw down handed to warp 0 (lw = nlev: none);
 // every level below the finest is fresh (seeded by its restriction), the
-// finest when `fresh`
-template <typename T>
-__device__ __forceinline__ void vcycle(const Lv<T>* L, int nlev, int lw, int nu1, int nu2, T* A, const T* f0,
+// finest when `fresh`.  A cluster (G = GClu) runs the levels below lx on all its
+// CTAs; the first CTA runs the others while the rest wait.
+template <typename T, typename G>
+__device__ __forceinline__ void vcycle(const Lv<T>* L, int nlev, int lx, int lw, int nu1, int nu2, T* A, const T* f0,
                                        bool fresh) {
+    constexpr bool CLU = std::is_same<G, GClu>::value;
     const bool seed = nu1 > 0;
     const int top = min(lw, nlev - 1);       // levels 0 .. top-1 run on the whole CTA
-    for (int l = 0; l < top; ++l) {
-        smooth<T, GCta>(L[l], nu1, (l > 0 || fresh) && seed);
-        resid_restrict<T, GCta>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
-    }
-    if (lw < nlev - 1) {
-        if (threadIdx.x < 32) {
-            for (int l = lw; l < nlev - 1; ++l) {
-                smooth<T, GWarp>(L[l], nu1, seed);
-                resid_restrict<T, GWarp>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
-            }
-            coarsest<T, GWarp>(L, nlev - 1, A, f0);
-            for (int l = nlev - 2; l >= lw; --l) prolong_smooth<T, GWarp>(L[l], L[l + 1], nu2);
+    if constexpr (CLU) {
+        for (int l = 0; l < lx; ++l) {
+            smooth<T, GClu>(L[l], nu1, (l > 0 || fresh) && seed);
+            resid_restrict<T, GClu>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
         }
-        __syncthreads();
-    } else {
-        coarsest<T, GCta>(L, nlev - 1, A, f0);
     }
-    for (int l = top - 1; l >= 0; --l) prolong_smooth<T, GCta>(L[l], L[l + 1], nu2);
+    const int l0 = CLU ? lx : 0;
+    if (!CLU || GClu::c().block_rank() == 0) {
+        for (int l = l0; l < top; ++l) {
+            smooth<T, GCta>(L[l], nu1, (l > 0 || fresh) && seed);
+            resid_restrict<T, GCta>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
+        }
+        if (lw < nlev - 1) {
+            if (threadIdx.x < 32) {
+                for (int l = lw; l < nlev - 1; ++l) {
+                    smooth<T, GWarp>(L[l], nu1, seed);
+                    resid_restrict<T, GWarp>(L[l], L[l + 1], nu1 > 0, l + 1 == nlev - 1, seed);
+                }
+                coarsest<T, GWarp>(L, nlev - 1, A, f0);
+                for (int l = nlev - 2; l >= lw; --l) prolong_smooth<T, GWarp>(L[l], L[l + 1], nu2);
+            }
+            __syncthreads();
+        } else {
+            coarsest<T, GCta>(L, nlev - 1, A, f0);
+        }
+        for (int l = top - 1; l >= l0; --l) prolong_smooth<T, GCta>(L[l], L[l + 1], nu2);
+    }
+    if constexpr (CLU) {
+        GClu::sync();
+        for (int l = lx - 1; l >= 0; --l) prolong_smooth<T, GClu>(L[l], L[l + 1], nu2);
+    }
 }
 
 // ||f - A dp||_inf on the finest (FP64) level after a cycle ending with a black
@@ -759,9 +788,9 @@ __device__ __forceinline__ void vcycle(const Lv<T>* L, int nlev, int lw, int nu1
 // red cells' scaled residual is g - dp with g the value that the next red
 // half-sweep would store: with `next` given, g is kept there, and the next
 // cycle starts from that half (see Cta::mg_solve) instead of sweeping.
-template <typename T>
-__device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool red_only, T* __restrict__ next,
-                                                         unsigned long long* red) {
+// Returns the thread's part of the maximum.
+template <typename T, typename G>
+__device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool red_only, T* __restrict__ next) {
     static_assert(Scaled<T>::value, "the mixed path's norm is its FP64 defect's");
     unsigned long long m = 0;
     const int nx = L.nx, nz = L.nz, hx = L.hx, H = L.H;
@@ -770,8 +799,8 @@ __device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool re
             const T* __restrict__ own = col ? L.db : L.dp;
             const T* __restrict__ oth = col ? L.dp : L.db;
             const T* __restrict__ D = L.D;
-            if (wide<T, GCta>(hx, H)) {
-                for (int c = 2 * threadIdx.x; c < H; c += 2 * blockDim.x) {
+            if (wide<T, G>(hx, H)) {
+                for (int c = 2 * G::rank(); c < H; c += 2 * G::size()) {
                     T g[2], d[2], x[2];
                     gs_vec<T>(c, fdiv(c, hx, L.mhx), nz, hx, H, col, L.f, L.c0, L.c1, L.c2, L.c3, L.q, oth, g);
                     ld_vec(D + col * H + c, d);
@@ -786,7 +815,7 @@ __device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool re
                 continue;
             }
 #pragma unroll 1
-            for (int c = threadIdx.x; c < H; c += blockDim.x) {
+            for (int c = G::rank(); c < H; c += G::size()) {
                 const int j = fdiv(c, hx, L.mhx);
                 const int i = 2 * (c - j * hx) + ((j + col) & 1);
                 const Nb s = nb_half(col, c, i, hx, H);
@@ -797,7 +826,7 @@ __device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool re
             }
         }
     } else {                                          // one level only: natural order
-        for (int c = threadIdx.x; c < L.nc; c += blockDim.x) {
+        for (int c = G::rank(); c < L.nc; c += G::size()) {
             const int j = fdiv(c, nx, L.mnx), i = c - j * nx;
             T v = L.f[c];
             if (i < nx - 1) v += L.c0[c] * L.dp[c + 1];
@@ -808,7 +837,7 @@ __device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool re
             m = b > m ? b : m;
         }
     }
-    return block_max(m, red);
+    return m;
 }
 
 // van Genuchten-Mualem closure at p < 0 (Eqs. Sw, sc_van, Krw) with
@@ -846,16 +875,20 @@ __device__ __forceinline__ void vg_eval(double a, double n, double m, double p, 
     dS = m * n * S * an / ((1.0 + an) * (-p));
 }
 
-// CTA-cooperative building blocks of one sample's solve.  Every method is
-// called by all threads of the CTA and ends with the CTA synchronised.
-template <typename TM, bool WC = false, int CL = 0>
+// Cooperative building blocks of one sample's solve on its CTA (G0 = GCta) or its
+// cluster of CTAs (GClu).  Every method is called by all threads of the group
+// and ends with the group synchronised; tid and nt count over the group.
+template <typename TM, bool WC = false, int CL = 0, typename G0 = GCta>
 struct Cta {
+    static constexpr bool CLU = std::is_same<G0, GClu>::value;   // the sample's group is a cluster
     static constexpr bool SC = Scaled<TM>::value;
     const FParams& P;
     Lv64* L64;
     Lv<TM>* LM;
     TM* Amat;
     unsigned long long* red;
+    unsigned long long (*cred)[8] = nullptr;   // cluster: the CTAs' maxima, two sets used in turn
+    int cpar = 0;
     double *f64, *dp64, *p, *thold, *Ks, *aa, *K, *th;
     double *nn, *mm, *trc, *tsc;          // closure 1: per-cell n, m, theta_r, theta_s
     int nx, nz, nc, nlev, tid, nt;
@@ -878,8 +911,31 @@ struct Cta {
             nn = mm = trc = tsc = nullptr;
         }
         nx = L64[0].nx; nz = L64[0].nz; nc = L64[0].nc; nlev = P.nlev;
-        tid = threadIdx.x; nt = blockDim.x;
+        tid = G0::rank(); nt = G0::size();
         h = P.h; t2h = P.two_over_h2; idt = P.inv_dt; tr = P.tr; ts = P.ts;
+    }
+
+    // maximum over the group, returned to every thread
+    __device__ __forceinline__ unsigned long long gmax(unsigned long long v) {
+        v = block_max(v, red);
+        if constexpr (CLU) {
+            auto c = GClu::c();
+            const int n = (int)c.num_blocks();
+            if ((int)threadIdx.x < n) *c.map_shared_rank(&cred[cpar][c.block_rank()], threadIdx.x) = v;
+            c.sync();
+            for (int k = 0; k < n; ++k) v = cred[cpar][k] > v ? cred[cpar][k] : v;
+            cpar ^= 1;                                 // the next but one write waits for the next barrier
+        }
+        return v;
+    }
+    // a level's threads in the set-up loops: a cluster's levels beyond lx belong
+    // to its first CTA (their arrays may be in its shared memory)
+    __device__ __forceinline__ bool mine(int l) const { return !CLU || l <= P.lx || tid < (int)blockDim.x; }
+    __device__ __forceinline__ int rank_on(int l) const { return CLU && l > P.lx ? (int)threadIdx.x : tid; }
+    __device__ __forceinline__ int size_on(int l) const { return CLU && l > P.lx ? (int)blockDim.x : nt; }
+    __device__ __forceinline__ void sync_on(int l) const {
+        if (!CLU || l <= P.lx) G0::sync();
+        else if (tid < (int)blockDim.x) __syncthreads();
     }
 
     // conductivity of cell q's soil at head pp (Dirichlet faces, QoI)
@@ -919,19 +975,21 @@ struct Cta {
                 tsc[q] = P.ts_in ? P.ts_in[o + q] : ts;
             }
         }
-        __syncthreads();
+        G0::sync();
         for (int i = tid; i < nx; i += nt) {
             int T = (nz - 1) * nx + i, B = i;
             F.Tbt[i] = t2h * k_at(T, P.p_top);
             F.Tbb[i] = t2h * k_at(B, P.p_bot);
         }
-        __syncthreads();
+        G0::sync();
         for (int l = 1; l < nlev; ++l) {
-            for (int I = tid; I < L64[l].nx; I += nt) {
-                L64[l].Tbt[I] = 0.25 * (0.5 * (L64[l - 1].Tbt[2 * I] + L64[l - 1].Tbt[2 * I + 1]));
-                L64[l].Tbb[I] = 0.25 * (0.5 * (L64[l - 1].Tbb[2 * I] + L64[l - 1].Tbb[2 * I + 1]));
+            if (mine(l)) {
+                for (int I = rank_on(l); I < L64[l].nx; I += size_on(l)) {
+                    L64[l].Tbt[I] = 0.25 * (0.5 * (L64[l - 1].Tbt[2 * I] + L64[l - 1].Tbt[2 * I + 1]));
+                    L64[l].Tbb[I] = 0.25 * (0.5 * (L64[l - 1].Tbb[2 * I] + L64[l - 1].Tbb[2 * I + 1]));
+                }
             }
-            __syncthreads();
+            sync_on(l);
         }
     }
 
@@ -946,7 +1004,7 @@ struct Cta {
                 thold[q] = pp < 0.0 ? r + (t - r) * vg_sat(aa[q], nn[q], mm[q], pp) : t;
             }
         }
-        __syncthreads();
+        G0::sync();
     }
 
     // a cell's correction at the start of a solve on the finest level: zero, or
@@ -987,7 +1045,7 @@ struct Cta {
                 }
             }
         }
-        __syncthreads();
+        G0::sync();
         for (int q = tid; q < nc; q += nt) {
             int j = fdiv(q, nx, F.mnx), i = q - j * nx;
             double kp = K[q];
@@ -996,7 +1054,7 @@ struct Cta {
             if (j < nz - 1) { double kn = K[q + nx]; F.Tz[q] = t2h * kp * kn / (kp + kn); }
             else F.Tz[q] = 0.0;
         }
-        __syncthreads();
+        G0::sync();
         unsigned long long m = 0;
         for (int q = tid; q < nc; q += nt) {
             int j = fdiv(q, nx, F.mnx), i = q - j * nx;
@@ -1030,14 +1088,14 @@ struct Cta {
             unsigned long long b = abs_bits(R);
             m = b > m ? b : m;
         }
-        const unsigned long long fb = block_max(m, red);
+        const unsigned long long fb = gmax(m);
         // coarse operators (Fig. diffUpscale)
         for (int l = 1; l < nlev; ++l) {
             const Lv64& Fl = L64[l - 1];
             const Lv64& Cl = L64[l];
             const Lv<TM>& Ml = LM[l];
             const int fx = Fl.nx;
-            for (int c = tid; c < Cl.nc; c += nt) {
+            for (int c = mine(l) ? rank_on(l) : Cl.nc; c < Cl.nc; c += size_on(l)) {
                 int J = fdiv(c, Cl.nx, Cl.mnx), I = c - J * Cl.nx;
                 int f00 = (2 * J) * fx + 2 * I, f01 = f00 + fx;
                 double cd = 0.25 * (Fl.Cdt[f00] + Fl.Cdt[f00 + 1] + Fl.Cdt[f01] + Fl.Cdt[f01 + 1]);
@@ -1060,7 +1118,7 @@ struct Cta {
                     Ml.q[sc] = (TM)(1.0f / (float)d);
                 }
             }
-            __syncthreads();
+            sync_on(l);
         }
         if (tid < 32) {
             const Lv64& Z = L64[nlev - 1];
@@ -1068,7 +1126,7 @@ struct Cta {
             if constexpr (SC) coarse_factor_warp<TM>(Z.nx, Z.nz, Z.Tx, Z.Tz, Z.D, Amat);
             else coarse_factor_warp<TM>(Z.nx, Z.nz, Mz.c0, Mz.c1, Mz.D, Amat);
         }
-        __syncthreads();
+        G0::sync();
         return fb;
     }
 
@@ -1078,7 +1136,7 @@ struct Cta {
     // (fresh: the red cells already hold their first half-sweep's values)
     __device__ void mgcycle(const TM* f0, bool fresh) {
         if constexpr (WC) gwalk<TM, GCta>(LM, 0, nlev, P.lw, P.nu1, P.nu2, P.gamma, Amat, f0, fresh);
-        else vcycle<TM>(LM, nlev, P.lw, P.nu1, P.nu2, Amat, f0, fresh);
+        else vcycle<TM, G0>(LM, nlev, P.lx, P.lw, P.nu1, P.nu2, Amat, f0, fresh);
     }
 
     // x += e (FP64, natural order += FP32 finest-level correction), then the
@@ -1092,7 +1150,7 @@ struct Cta {
             const int j = fdiv(q, nx, mnx), i = q - j * nx;
             x[q] += (double)e[sidx(M0, i, j)];
         }
-        __syncthreads();
+        G0::sync();
     }
 
     // FP64 defect r = f - A x of the finest operator, stored as the next FP32
@@ -1146,14 +1204,14 @@ struct Cta {
             if constexpr (SC) {
                 if (cyc > 0) {
                     if (keep) {
-                        if (tid == 0) { TM* t = LM[0].dp; LM[0].dp = LM[0].alt; LM[0].alt = t; }
+                        if (threadIdx.x == 0) { TM* t = LM[0].dp; LM[0].dp = LM[0].alt; LM[0].alt = t; }
                         __syncthreads();
                     }
                     fresh = keep;
                 }
                 mgcycle((const TM*)f64, fresh);
                 ++cyc;
-                rb = resid_norm<TM>(M0, P.nu2 > 0 && nlev > 1, keep ? M0.alt : nullptr, red);
+                rb = gmax(resid_norm<TM, G0>(M0, P.nu2 > 0 && nlev > 1, keep ? M0.alt : nullptr));
             } else {
                 for (int in = 0; in < P.mixed_inner && cyc < P.mg_maxit; ++in) {
                     mgcycle(nullptr, in == 0);
@@ -1162,7 +1220,7 @@ struct Cta {
                 // dp += e in FP64, then the FP64 defect: stopping norm and the
                 // next FP32 right-hand side
                 add_correction(dp64, M0.dp);
-                rb = block_max(defect(f64, dp64, L64[0].Tx, L64[0].Tz, L64[0].D, M0.q, M0.f, M0.dp), red);
+                rb = gmax(defect(f64, dp64, L64[0].Tx, L64[0].Tz, L64[0].D, M0.q, M0.f, M0.dp));
             }
             if (rb > INF_BITS - 1) { mg_tot += cyc; return false; }
             rn = __longlong_as_double((long long)rb);
@@ -1170,7 +1228,7 @@ struct Cta {
         if constexpr (SC) {
             if (cyc == 0) {                           // nothing to solve: the correction is zero, not its seed
                 for (int c = tid; c < M0.H; c += nt) M0.dp[c] = TM(0);
-                __syncthreads();
+                G0::sync();
             }
         }
         mg_tot += cyc;
@@ -1203,7 +1261,7 @@ struct Cta {
                 unsigned long long b = abs_bits(d);
                 dm = b > dm ? b : dm;
             }
-            const unsigned long long db = block_max(dm, red);
+            const unsigned long long db = gmax(dm);
             ++k;
             ++pic_tot;
             if (db > INF_BITS - 1) { status = RICH_NONFINITE; alive = false; break; }
@@ -1609,6 +1667,33 @@ __device__ __forceinline__ void init_levels(const FParams& P, char* slot, unsign
     __syncthreads();
 }
 
+// one sample on its group, results to the caller's arrays; a group holds `sms`
+// CTAs (the time it is charged)
+template <typename C_t>
+__device__ __forceinline__ void solve_sample(C_t& C, const FParams& P, int s, int sms) {
+    const int nc = C.nc, tid = C.tid, nt = C.nt;
+    const unsigned long long t0 = globaltimer_ns();
+    C.setup(s);
+    int status = RICH_OK, maxpic = 0;
+    bool alive = true;
+    long long pic_tot = 0, mg_tot = 0;
+    for (int step = 0; step < P.nsteps && alive; ++step)
+        alive = C.time_step(pic_tot, mg_tot, maxpic, status);
+    if (tid < 32) {
+        const double q = C.qoi_warp0();
+        if (tid == 0) {
+            P.qoi[s] = alive ? q : __longlong_as_double(0x7FF8000000000000ll);
+            if (P.status) P.status[s] = status;
+            if (P.pic_total) P.pic_total[s] = pic_tot;
+            if (P.mg_total) P.mg_total[s] = mg_tot;
+            if (P.maxpic) P.maxpic[s] = maxpic;
+            if (P.t_ns) P.t_ns[s] = (int64_t)(globaltimer_ns() - t0) * sms;
+        }
+    }
+    if (P.p_final)
+        for (int q = tid; q < nc; q += nt) P.p_final[(size_t)s * nc + q] = C.p[q];
+}
+
 template <typename TM, int NT, bool WC, int CL>
 __global__ void __launch_bounds__(NT, NT == 32 ? 32 : NT <= 128 ? 8 : NT <= 256 ? 4 : NT == 512 ? 2 : 1)
 k_fused(const FParams P) {
@@ -1620,34 +1705,51 @@ k_fused(const FParams P) {
     char* slot = P.scratch + (size_t)blockIdx.x * P.slot_bytes;
     init_levels<TM>(P, slot, smraw, L64, LM);
     Cta<TM, WC, CL> C(P, slot, L64, LM, reinterpret_cast<TM*>(smraw), red);
-    const int nc = C.nc, tid = C.tid, nt = C.nt;
+    const int tid = C.tid;
     for (;;) {
         if (tid == 0) s_sample = atomicAdd(P.queue, 1);
         __syncthreads();
         const int s = s_sample;
         __syncthreads();
         if (s >= P.S) break;
-        const unsigned long long t0 = globaltimer_ns();
-        C.setup(s);
-        int status = RICH_OK, maxpic = 0;
-        bool alive = true;
-        long long pic_tot = 0, mg_tot = 0;
-        for (int step = 0; step < P.nsteps && alive; ++step)
-            alive = C.time_step(pic_tot, mg_tot, maxpic, status);
-        if (tid < 32) {
-            const double q = C.qoi_warp0();
-            if (tid == 0) {
-                P.qoi[s] = alive ? q : __longlong_as_double(0x7FF8000000000000ll);
-                if (P.status) P.status[s] = status;
-                if (P.pic_total) P.pic_total[s] = pic_tot;
-                if (P.mg_total) P.mg_total[s] = mg_tot;
-                if (P.maxpic) P.maxpic[s] = maxpic;
-                if (P.t_ns) P.t_ns[s] = (int64_t)(globaltimer_ns() - t0);
-            }
-        }
-        if (P.p_final)
-            for (int q = tid; q < nc; q += nt) P.p_final[(size_t)s * nc + q] = C.p[q];
+        solve_sample(C, P, s, 1);
         __syncthreads();
+    }
+}
+
+// The same with a cluster of CTAs, each on an SM of its own, per sample: a batch
+// with fewer samples than half the SMs leaves the others idle, and a large grid's
+// half-sweeps are long enough to pay for a cluster barrier (about a microsecond
+// with the reads that follow it) after each.  Fine levels run on all CTAs, their
+// arrays in the slot; the first CTA runs the rest (vcycle).  256^2 x 24 samples,
+// mixed: 247 -> 86 ms; one 64^2 sample, FP64: 146 -> 104 ms.
+constexpr int CLUSTER_THREADS = 512;
+template <typename TM, int CL>
+__global__ void __launch_bounds__(CLUSTER_THREADS, 1)
+k_fused_cluster(const FParams P) {
+    extern __shared__ unsigned char smraw[];
+    __shared__ unsigned long long red[33];
+    __shared__ unsigned long long cred[2][8];
+    __shared__ int s_sample;
+    __shared__ Lv64 L64[MAXL];
+    __shared__ Lv<TM> LM[MAXL];
+    auto c = GClu::c();
+    const int n = (int)c.num_blocks();
+    char* slot = P.scratch + (size_t)(blockIdx.x / n) * P.slot_bytes;
+    init_levels<TM>(P, slot, smraw, L64, LM);
+    Cta<TM, false, CL, GClu> C(P, slot, L64, LM, reinterpret_cast<TM*>(smraw), red);
+    C.cred = cred;
+    c.sync();                                         // every CTA runs before its memory is written to
+    for (;;) {
+        if (C.tid == 0) {
+            const int s = atomicAdd(P.queue, 1);
+            for (int k = 0; k < n; ++k) *c.map_shared_rank(&s_sample, k) = s;
+        }
+        c.sync();
+        const int s = s_sample;
+        if (s >= P.S) break;
+        solve_sample(C, P, s, n);
+        c.sync();
     }
 }
 
@@ -1693,5 +1795,24 @@ void launch_shapes(const FParams& P, int grid, size_t smem, int nt, cudaStream_t
         if (wc) k_fused<TM, 512, true, CL><<<grid, 512, smem, st>>>(P);
         else k_fused<TM, 512, false, CL><<<grid, 512, smem, st>>>(P);
     }
+}
+
+// clusters of n CTAs: fit != null asks how many the GPU holds at a time, else
+// `clusters` of them are launched
+template <typename TM, int CL>
+int cluster_call(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(clusters * n)); cfg.blockDim = dim3(CLUSTER_THREADS);
+    cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = at; cfg.numAttrs = 1;
+    if (fit) {
+        if (int e = allow_dyn_smem((const void*)k_fused_cluster<TM, CL>, smem)) return e;
+        RICH_CUDA(cudaOccupancyMaxActiveClusters(fit, k_fused_cluster<TM, CL>, &cfg));
+        return 0;
+    }
+    RICH_CUDA(cudaLaunchKernelEx(&cfg, k_fused_cluster<TM, CL>, P));
+    return 0;
 }
 }  // namespace
