@@ -293,6 +293,35 @@ FXD double fx_exp(double x) {
     return fx_to_double(v, n);
 }
 
+// a / b to 0.51 units in the last place where both are positive and normal and
+// the quotient is well inside the normal range (all else: the FP64 division,
+// which holds its pipe for about 9 multiply-adds, two to four of them a cell and
+// Picard iteration: 608 samples on 128^2 are 4.8 % faster in mixed precision and
+// 2.7 % in FP64): a 23-bit reciprocal of b and its third-order correction
+FX double fx_div(double a, double b) {
+    const unsigned long long ba = double_bits(a), bb = double_bits(b), one = 1ull << 52;
+    const int ea = (int)(ba >> 52), eb = (int)(bb >> 52), ex = ea - eb + 1023;
+    if ((unsigned)(ea - 1) >= 2046u || (unsigned)(eb - 1) >= 2046u || ex < 8 || ex > 2038) return a / b;
+    const unsigned long long B = (bb | one) << 11;           // [2^63, 2^64): b's mantissa in Q63
+    const unsigned int fb = 0x3F800000u | ((unsigned int)(B >> 40) & 0x7FFFFFu);
+#ifdef __CUDA_ARCH__
+    const unsigned int fy = __float_as_uint(__frcp_rn(__uint_as_float(fb)));
+#else
+    float f; memcpy(&f, &fb, 4); f = 1.0f / f;
+    unsigned int fy; memcpy(&fy, &f, 4);
+#endif
+    const uint32_t Y = fy == 0x3F800000u ? 0x7FFFFFFFu : ((fy & 0x7FFFFFu) | 0x800000u) << 7;     // 1/b in Q31
+    // d = 1 - b Y in Q62, |d| < 2^-21
+    const long long d = (long long)((1ull << 62) - ((B >> 32) * Y + (((B & 0xFFFFFFFFull) * Y) >> 32)));
+    const long long dh = d >> 16;
+    const long long c = d + ((dh * dh) >> 30);
+    const long long y = ((long long)Y << 31) + rmul(c, (long long)Y << 31);
+    unsigned long long q = (unsigned long long)rmul((long long)((ba & (one - 1)) | one) << 9, y);   // a/b in Q61
+    int n = ex - 1023;
+    if (!(q >> 61)) { q <<= 1; --n; }
+    return fx_to_double(q << 1, n);
+}
+
 // e^(y 2^-F), |y 2^-F| < 512, as v 2^n
 template <int F>
 FXD unsigned long long exp_fixed(long long y, int& n) {

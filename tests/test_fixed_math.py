@@ -13,6 +13,7 @@ SRC = r"""
 #include "fixed.cuh"
 using namespace rich_fx;
 extern "C" void t_exp(int n, const double* x, double* y) { for (int i = 0; i < n; ++i) y[i] = fx_exp(x[i]); }
+extern "C" void t_div(int n, const double* a, const double* b, double* q) { for (int i = 0; i < n; ++i) q[i] = fx_div(a[i], b[i]); }
 extern "C" void t_vg(int k, const double* ap, const double* n, const double* m, int* ok, double* s, double* kr, double* d) {
     for (int i = 0; i < k; ++i) { VgLog o; ok[i] = vg_log(ap[i], n[i], m[i], o); if (ok[i]) { s[i] = vg_s(o); vg_k(o, kr[i], d[i]); } }
 }
@@ -53,6 +54,27 @@ def test_exp_is_within_six_tenths_of_a_unit(lib):
         f = np.isfinite(rounded) & (rounded > 1e-300)
         assert (np.abs(y[f] - want[f]) / np.spacing(rounded[f])).max() < 0.6
         assert np.array_equal(y[x == 0], np.ones(2)) and y[x == -800.0] == 0
+
+
+def test_division_is_within_six_tenths_of_a_unit(lib):
+    """Mantissas at both ends and throughout, quotients over the whole range;
+    what is not positive, normal or in range gives the division's own bits."""
+    g = np.random.default_rng(3)
+    k = 60000
+    a, b = (1 + g.random(k)) * 2.0 ** g.integers(-400, 400, k), (1 + g.random(k)) * 2.0 ** g.integers(-400, 400, k)
+    b[:1000] = np.nextafter(2.0, 0) * 2.0 ** g.integers(-9, 9, 1000)
+    b[1000:2000] = 1 + 2.0 ** -52 * g.integers(0, 9, 1000)
+    a[2000:3000] = b[2000:3000]
+    special = np.array([0.0, -0.0, 1.0, -3.0, np.inf, -np.inf, np.nan, 5e-324, 2e-308, 1.7e308])
+    sa, sb = (v.ravel() for v in np.meshgrid(special, special))
+    q, sq = np.empty(k), np.empty(len(sa))
+    lib.t_div(k, dp(a), dp(b), dp(q))
+    want = a.astype(np.longdouble) / b.astype(np.longdouble)
+    assert (np.abs(q - want) / np.spacing(a / b)).max() < 0.6
+    assert np.array_equal(q[2000:3000], np.ones(1000))
+    lib.t_div(len(sa), dp(sa), dp(sb), dp(sq))
+    with np.errstate(all="ignore"):
+        assert np.allclose(sq, sa / sb, rtol=2.3e-16, atol=0, equal_nan=True)
 
 
 def test_van_genuchten_matches_the_library_functions(lib):
