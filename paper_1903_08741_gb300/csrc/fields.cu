@@ -12,8 +12,9 @@
 // third runs half of them.  Within the transforms frequencies stay in
 // bit-reversed order; the filter is laid out in it.  In FP64, one kernel a pass
 // (noise, row and column transforms both ways, filter, window), 512 draws of a
-// 128^2 pair took 63.1 ms, now 9.4; 64 of a 32^2 pair 477 us, now 103; 512
-// couples of five 64^2 fields 13.1 ms, now 3.7.
+// 128^2 pair took 63.1 ms, now 8.7; 64 of a 32^2 pair 477 us, now 94; 512
+// couples of five 64^2 fields 13.1 ms, now 2.0.  What is left is the 32-bit multiply
+// and add pipes (the first kernel issues on 67 % of its cycles).
 // White noise: Philox4x32-10 (Salmon et al., SC'11) implemented from its
 // definition, key = (seed low word, seed high word ^ level), counter = (cell
 // pair, field, sample low, sample high), two uniforms -> Box-Muller.
@@ -32,10 +33,9 @@ __device__ __forceinline__ void philox10(uint32_t c[4], uint32_t k0, uint32_t k1
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
         if (r) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
-        uint32_t hi0 = __umulhi(0xD2511F53u, c[0]), lo0 = 0xD2511F53u * c[0];
-        uint32_t hi1 = __umulhi(0xCD9E8D57u, c[2]), lo1 = 0xCD9E8D57u * c[2];
-        uint32_t n0 = hi1 ^ c[1] ^ k0, n2 = hi0 ^ c[3] ^ k1;
-        c[0] = n0; c[1] = lo1; c[2] = n2; c[3] = lo0;
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c[0], p1 = (uint64_t)0xCD9E8D57u * c[2];
+        const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c[1] ^ k0, n2 = (uint32_t)(p0 >> 32) ^ c[3] ^ k1;
+        c[0] = n0; c[1] = (uint32_t)p1; c[2] = n2; c[3] = (uint32_t)p0;
     }
 }
 
@@ -157,9 +157,9 @@ struct PackTr {
     double im_lo, im_span;
 };
 
-__device__ __forceinline__ double uniform_of(double z, double inv_sigma, double lo, double span) {
-    double gg = z * inv_sigma;
-    return lo + span * 0.5 * erfc(-gg / sqrt(2.0));
+__device__ __forceinline__ double uniform_of(double z, double inv_sigma, double lo, double span,
+                                             const PhiEntry* __restrict__ tab) {
+    return lo + span * normal_cdf(z * inv_sigma, tab);
 }
 
 // ---------------------------------------------------------------- transforms
@@ -235,9 +235,12 @@ __device__ __forceinline__ void inverse_passes(fx2* sm, int logn, int loglpb, in
 
 constexpr int FT = 256;                     // threads of the transform kernels
 
-// the noise of the torus (COARSE: half the 2x2 sums of the torus of twice the
-// sides, so that it stays standard normal: Appendix A, Eq. averaging) and its row
-// transforms, frequencies bit-reversed; 2^loglpb rows a block
+// the noise of the torus and its row transforms, frequencies bit-reversed;
+// 2^loglpb rows a block.  The coarse member's noise is half the 2x2 sums of the
+// torus of twice the sides (it stays standard normal: Appendix A, Eq. averaging):
+// a block of two rows or more leaves it in `coarse` for the LOADED launch (drawing
+// it again there: 512 couples of five 64^2 fields 3.7 ms, so 2.0); where only one
+// row of 8192 fits, the COARSE launch does draw it again.
 // (first sample = *first_dev + first when first_dev is given: a captured CUDA
 // graph can advance the sample range between replays)
 struct RowArgs {
@@ -251,9 +254,11 @@ struct RowArgs {
     const NormTab* norm;
     const cw* tw;
     fx2* out;
+    fx2* coarse;
 };
+enum { FINE, COARSE, LOADED };
 
-template <bool COARSE>
+template <int SRC>
 __global__ void __launch_bounds__(FT, 3) k_noise_rows(const RowArgs A) {
     extern __shared__ fx2 sm[];
     const int logn = A.logpx, n = 1 << logn, lpb = 1 << A.loglpb;
@@ -265,18 +270,22 @@ __global__ void __launch_bounds__(FT, 3) k_noise_rows(const RowArgs A) {
         philox10(c, k0, k1);
         normal_pair(c[0], c[1], c[2], c[3], A.norm, y0, y1);
     };
-    const int lw = COARSE ? logn : logn - 1;          // a thread's unit: a point; two neighbours
+    const int lw = SRC == FINE ? logn - 1 : logn;     // a thread's unit: two neighbours; a point
     for (int it = threadIdx.x; it < lpb << lw; it += FT) {
         const int l = it >> lw, x = it & ((1 << lw) - 1);
         const long long line = line0 + l;
         if (line >= A.lines) break;
+        if (SRC == LOADED) {
+            sm[at<false>(l, x, logn, 0)] = A.coarse[(line << logn) + x];
+            continue;
+        }
         const uint64_t sample = (uint64_t)(first + (line >> A.logpz));
         const uint32_t row = (uint32_t)(line & ((1ll << A.logpz) - 1));
         long long y[2][2] = {};
 #pragma unroll 1
         for (int f = 0; f < (A.im ? 2 : 1); ++f) {
             long long a, b;
-            if (COARSE) {
+            if (SRC == COARSE) {
                 long long c, d;
                 draw(((2 * row) << logn) + x, f, sample, a, b);
                 draw(((2 * row + 1) << logn) + x, f, sample, c, d);
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(FT, 3) k_noise_rows(const RowArgs A) {
             }
             if (f) { y[1][0] = a; y[1][1] = b; } else { y[0][0] = a; y[0][1] = b; }
         }
-        if (COARSE) {
+        if (SRC == COARSE) {
             sm[at<false>(l, x, logn, 0)] = fx2{y[0][0], y[1][0]};
         } else {
             sm[at<false>(l, 2 * x, logn, 0)] = fx2{y[0][0], y[1][0]};
@@ -294,6 +303,16 @@ __global__ void __launch_bounds__(FT, 3) k_noise_rows(const RowArgs A) {
         }
     }
     __syncthreads();
+    if (SRC == FINE && A.coarse) {
+        for (int t = threadIdx.x; t < n << A.loglpb >> 2; t += FT) {
+            const int l = 2 * (t >> (logn - 1)), x = 2 * (t & ((n >> 1) - 1));
+            if (line0 + l >= A.lines) break;
+            const fx2 v = sm[at<false>(l, x, logn, 0)] + sm[at<false>(l, x + 1, logn, 0)] +
+                          sm[at<false>(l + 1, x, logn, 0)] + sm[at<false>(l + 1, x + 1, logn, 0)];
+            A.coarse[(((line0 + l) >> 1) << (logn - 1)) + (x >> 1)] = fx2{(v.re + 1) >> 1, (v.im + 1) >> 1};
+        }
+        __syncthreads();
+    }
     for (int b = 0; b < logn;) {
         const int w = pass_bits(logn, b);
         any_pass<false, false, false>(w, sm, logn, A.loglpb, b, A.tw);
@@ -332,7 +351,7 @@ k_columns(int logpx, int logpz, int loglpb, int nz, const cw* __restrict__ tw, c
 __global__ void __launch_bounds__(FT, 3)
 k_rows_window(long long lines, int logpx, int logpz, int loglpb, int lognx, int lognz, const cw* __restrict__ tw,
               const int* __restrict__ colsh, double scale, const fx2* __restrict__ data, double inv_sigma, PackTr tr,
-              double* lk, double* al) {
+              const PhiEntry* __restrict__ tab, double* lk, double* al) {
     extern __shared__ fx2 sm[];
     const int n = 1 << logpx;
     const long long line0 = (long long)blockIdx.x << loglpb;
@@ -355,8 +374,8 @@ k_rows_window(long long lines, int logpx, int logpz, int loglpb, int lognx, int 
         const long long g = ((line0 + l) << lognx) + i;
         const fx2 v = sm[at<false>(l, i, logpx, 0)];
         const double re = (double)v.re * scale;
-        lk[g] = tr.re_uniform ? uniform_of(re, inv_sigma, tr.re_a, tr.re_b) : re + tr.re_a;
-        if (al) al[g] = uniform_of((double)v.im * scale, inv_sigma, tr.im_lo, tr.im_span);
+        lk[g] = tr.re_uniform ? uniform_of(re, inv_sigma, tr.re_a, tr.re_b, tab) : re + tr.re_a;
+        if (al) al[g] = uniform_of((double)v.im * scale, inv_sigma, tr.im_lo, tr.im_span, tab);
     }
 }
 
@@ -553,12 +572,14 @@ static int ensure_work(rich_ctx* ctx, size_t bytes) {
     return 0;
 }
 
+constexpr int PAIR_LOG = 12;                // two rows of 4096 points fit a block, two of 8192 do not
+
 // log2 of the lines of n points a block takes: 2048 points (8 a thread, 36 KB of
 // shared memory), fewer while that leaves SMs without a block; at least `least`
-// where 128 KB hold them, and no more than `most`
-static int log_lines(const rich_ctx* ctx, int logn, long long lines, int least, int most) {
+// where `bytes` hold them, and no more than `most`
+static int log_lines(const rich_ctx* ctx, int logn, long long lines, int least, int most, long long bytes) {
     int l = std::max(11 - logn, least);
-    while (l > 0 && (16ll << (logn + l)) > (64 << 10)) --l;
+    while (l > 0 && (16ll << (logn + l)) > bytes) --l;
     while (l > least && logn + l > 8 && (lines >> l) < ctx->sm_count) --l;
     return std::min(l, most);
 }
@@ -576,35 +597,41 @@ static int allow_smem(K kernel, size_t bytes) {
 
 // FFT-MA of one packed pair of fields for cs samples in `work` ([cs][pz][px]):
 // the window's nx x nz cells to re and im (im null: that lane is not wanted).
-// coarse: the noise is that of the torus of twice the sides, upscaled.
+// A pair's first member leaves the second one's noise in `noise` (PAIR_FINE; see
+// k_noise_rows).
+enum { SINGLE, PAIR_FINE, PAIR_COARSE };
 static int fftma(rich_ctx* ctx, const rich_spectrum* sp, fx2* work, int cs, uint64_t seed, uint32_t level,
-                 int64_t first, const int64_t* first_dev, uint32_t fld0, bool coarse, int nx, int nz,
+                 int64_t first, const int64_t* first_dev, uint32_t fld0, int role, fx2* noise, int nx, int nz,
                  double inv_sigma, const PackTr& tr, double* re, double* im, cudaStream_t st) {
     const int lx = ilog2(sp->px), lz = ilog2(sp->pz), lnx = ilog2(nx), lnz = ilog2(nz);
     RowArgs A{};
     A.lines = (long long)cs << lz;
-    A.logpx = lx; A.logpz = lz; A.loglpb = log_lines(ctx, lx, A.lines, 0, 11);
+    A.logpx = lx; A.logpz = lz; A.loglpb = log_lines(ctx, lx, A.lines, role == PAIR_FINE ? 1 : 0, 11, 128 << 10);
     A.seed = seed; A.level = level; A.fld0 = fld0; A.im = im != nullptr; A.first = first; A.first_dev = first_dev;
     A.norm = (const NormTab*)sp->norm; A.tw = (const cw*)sp->twx; A.out = work;
+    // (the finer torus has rows of twice this one's length)
+    const bool shared = role == PAIR_FINE ? A.loglpb > 0 : role == PAIR_COARSE && lx + 1 <= PAIR_LOG;
+    A.coarse = shared ? noise : nullptr;
     size_t smem = row_smem(lx, A.loglpb);
-    auto* rows = coarse ? k_noise_rows<true> : k_noise_rows<false>;
+    auto* rows = role != PAIR_COARSE ? k_noise_rows<FINE> : shared ? k_noise_rows<LOADED> : k_noise_rows<COARSE>;
     if (int e = allow_smem(rows, smem)) return e;
     rich_count_launch();
     rows<<<(unsigned)((A.lines + (1ll << A.loglpb) - 1) >> A.loglpb), FT, smem, st>>>(A);
     // columns: eight side by side fill a 128-byte line
-    const int lc = log_lines(ctx, lz, (long long)cs << lx, std::min(3, lx), lx);
+    const int lc = log_lines(ctx, lz, (long long)cs << lx, std::min(3, lx), lx, 64 << 10);
     smem = sizeof(fx2) << (lz + lc);
     if (int e = allow_smem(k_columns, smem)) return e;
     rich_count_launch();
     k_columns<<<(unsigned)((long long)cs << (lx - lc)), FT, smem, st>>>(lx, lz, lc, nz, (const cw*)sp->twz,
                                                                        (const wq*)sp->filt, work);
     const long long wl = (long long)cs << lnz;
-    const int lw = log_lines(ctx, lx, wl, 0, 11);
+    const int lw = log_lines(ctx, lx, wl, 0, 11, 128 << 10);
     smem = row_smem(lx, lw);
     if (int e = allow_smem(k_rows_window, smem)) return e;
     rich_count_launch();
     k_rows_window<<<(unsigned)((wl + (1ll << lw) - 1) >> lw), FT, smem, st>>>(
-        wl, lx, lz, lw, lnx, lnz, (const cw*)sp->twx, sp->colsh, sp->scale, work, inv_sigma, tr, re, im);
+        wl, lx, lz, lw, lnx, lnz, (const cw*)sp->twx, sp->colsh, sp->scale, work, inv_sigma, tr,
+        ((const NormTab*)sp->norm)->phi, re, im);
     RICH_CUDA(cudaGetLastError());
     return 0;
 }
@@ -653,8 +680,8 @@ static int packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int nz, u
             const bool im = P.out_im != nullptr;
             double* wl = coarsen ? bl[0] : P.out_re + (size_t)s0 * nx * nz;
             double* wa = !im ? nullptr : coarsen ? ba[0] : P.out_im + (size_t)s0 * nx * nz;
-            if (int e = fftma(ctx, sp, work, cs, fd->seed, level, first + s0, first_dev, P.fld0, false, nx, nz,
-                              inv_sigma, P.tr, wl, wa, st))
+            if (int e = fftma(ctx, sp, work, cs, fd->seed, level, first + s0, first_dev, P.fld0, SINGLE, nullptr, nx,
+                              nz, inv_sigma, P.tr, wl, wa, st))
                 return e;
             int cx = nx, cz = nz, cur = 0;
             for (int c = 0; c < coarsen; ++c) {
@@ -728,10 +755,11 @@ static int pair_packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int 
     spectrum_on(ctx, px, pz, 1.0 / nz, fd, st, &spf, nullptr);
     spectrum_on(ctx, px / 2, pz / 2, 2.0 / nz, fd, st, &spc, nullptr);
     const int npf = px * pz;
-    const size_t per = (size_t)npf * sizeof(fx2);
+    const size_t per = (size_t)(npf + npf / 4) * sizeof(fx2);
     const int cap = (int)std::min<size_t>((size_t)S, std::max<size_t>(1, CHUNK_BYTES / per));
     if (int e = ensure_work(ctx, per * cap)) return e;
     fx2* work = (fx2*)ctx->field_work;         // the two members take turns
+    fx2* noise = work + (size_t)npf * cap;
     const double inv_sigma = 1.0 / sqrt(fd->sigma2);
     const int ncx = nx / 2, ncz = nz / 2;
     for (int s0 = 0; s0 < S; s0 += cap) {
@@ -739,11 +767,11 @@ static int pair_packs_device(rich_ctx* ctx, const rich_field_t* fd, int nx, int 
         for (int k = 0; k < npk; ++k) {
             const PairPack& P = pk[k];
             const size_t of = (size_t)s0 * nx * nz, oc = (size_t)s0 * ncx * ncz;
-            if (int e = fftma(ctx, spf, work, cs, fd->seed, level, first + s0, nullptr, P.fld0, false, nx, nz,
-                              inv_sigma, P.tr, P.f_re + of, P.f_im ? P.f_im + of : nullptr, st))
+            if (int e = fftma(ctx, spf, work, cs, fd->seed, level, first + s0, nullptr, P.fld0, PAIR_FINE, noise,
+                              nx, nz, inv_sigma, P.tr, P.f_re + of, P.f_im ? P.f_im + of : nullptr, st))
                 return e;
-            if (int e = fftma(ctx, spc, work, cs, fd->seed, level, first + s0, nullptr, P.fld0, true, ncx, ncz,
-                              inv_sigma, P.tr, P.c_re + oc, P.c_im ? P.c_im + oc : nullptr, st))
+            if (int e = fftma(ctx, spc, work, cs, fd->seed, level, first + s0, nullptr, P.fld0, PAIR_COARSE, noise,
+                              ncx, ncz, inv_sigma, P.tr, P.c_re + oc, P.c_im ? P.c_im + oc : nullptr, st))
                 return e;
         }
     }

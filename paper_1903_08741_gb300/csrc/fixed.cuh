@@ -138,7 +138,9 @@ FX int pass_bits(int logn, int b0) {
 // unit circle at 256ths of a turn
 struct LogEntry { long long l57; int inv; int pad; };
 constexpr long long LN2_57 = 0x162E42FEFA39EF3ll >> 0;      // ln 2 in Q57
-struct NormTab { LogEntry lg[256]; cw cs[256]; };
+struct PhiEntry { long long phi, c[4]; int b[4], e, pad; };    // Phi_k = phi 2^-62 2^e
+constexpr int PHI_SIDE = 256;
+struct NormTab { LogEntry lg[256]; cw cs[256]; PhiEntry phi[2 * PHI_SIDE + 1]; };
 
 FX int clz64(unsigned long long x) {
 #ifdef __CUDA_ARCH__
@@ -156,16 +158,15 @@ FX unsigned long long uniform54(uint32_t hi, uint32_t lo) {
 }
 
 // log(1 + r) in Q70 for r in Q70, |r| <= 2^-8: r - r^2 P(r), Taylor to r^8
-// (remainder 2^-67 of r); the factors of r^3 and on in 32 bits
+// (remainder 2^-67 of r); the factors of r^3 and on from 32-bit halves (2^-63)
 FX long long log1p70(long long r) {
     const long long r62 = r >> 8;
-    const int r31 = (int)(r >> 39);
-    int t = (int)(0x80000000u / 7) - (int)(wide(0x10000000, r31) >> 31);
-    t = (int)(0x80000000u / 6) - (int)(wide(t, r31) >> 31);
-    t = (int)(0x80000000u / 5) - (int)(wide(t, r31) >> 31);
-    long long p = (1ll << 60) - rmul(r62, (long long)t << 31);
-    p = (1ll << 62) / 3 - rmul(r62, p);
-    p = (1ll << 61) - rmul(r62, p);
+    const int r39 = (int)(r >> 31);
+    int t = (int)(0x80000000u / 7) - (int)(wide(0x10000000, r39) >> 39);
+    t = (int)(0x80000000u / 6) - (int)(wide(t, r39) >> 39);
+    t = (int)(0x80000000u / 5) - (int)(wide(t, r39) >> 39);
+    t = 0x20000000 - (int)(wide(t, r39) >> 39);
+    const long long p = (1ll << 61) - rmul(r62, (1ll << 62) / 3 - (wide(t, r39) >> 8));
     return r - rmul(rmul(r, p), r62);
 }
 
@@ -377,13 +378,62 @@ FXD void vg_k(const VgLog& o, double& krw, double& d) {
     d = exp_fixed<53>(q - (o.l1 >> 4));
 }
 
+// The normal distribution function about z_k = k/64, |z_k| <= 4: Phi(z_k + d) =
+// Phi_k (1 + s), s the Taylor series of degree 8 (remainder 2^-63), its n-th
+// coefficient phi_k He_{n-1}(z_k) (-1)^(n-1) / (n! Phi_k) in units of 2^-7n; those
+// from the fifth on in 32 bits (all Q62).  erfc held the FP64 pipe for 78
+// operations a value, most of the last transform kernel's time.
+FX double normal_cdf(double z, const PhiEntry* tab) {
+    const unsigned long long bits = double_bits(z), one = 1ull << 52;
+    const int e = (int)(bits >> 52 & 0x7FF) - 1023;
+    if (e > 1) return 0.5 * erfc(-z / sqrt(2.0));            // |z| >= 4, NaN
+    const unsigned long long m = (bits & (one - 1)) | one;
+    long long q = e >= -7 ? (long long)(m << (e + 7)) : e >= -60 ? (long long)(m >> -(e + 7)) : 0;   // |z| in Q59
+    if (bits >> 63) q = -q;
+    const int k = (int)((q + (1ll << 52)) >> 53);
+    const long long d = (q - ((long long)k << 53)) << 10;    // 2^7 (z - z_k) in Q62
+    const PhiEntry t = tab[k + PHI_SIDE];
+    const int d31 = (int)((d - (d >> 62)) >> 31);            // (1 as the largest number below)
+    int b = t.b[3];
+    b = t.b[2] + (int)(wide(b, d31) >> 31);
+    b = t.b[1] + (int)(wide(b, d31) >> 31);
+    b = t.b[0] + (int)(wide(b, d31) >> 31);
+    long long s = t.c[3] + (wide(b, d31) >> 31);
+    s = t.c[2] + rmul(s, d);
+    s = t.c[1] + rmul(s, d);
+    s = t.c[0] + rmul(s, d);
+    s = rmul(s, d);
+    unsigned long long v = (unsigned long long)(t.phi + rmul(t.phi, s));
+    int n = t.e;
+    if (v >> 63) { v >>= 1; ++n; }
+    else if (!(v >> 62)) { v <<= 1; --n; }
+    return fx_to_double(v, n);
+}
+
 // the tables, from the host's long double functions
 inline long long to_q(long double v, int bits) { return (long long)llrintl(ldexpl(v, bits)); }
 inline cw circle_point(long long k, long long n) {
     const long double t = 2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)n;
     return cw{split_w(to_q(cosl(t), 62)), split_w(to_q(sinl(t), 62))};
 }
+inline void make_phi(PhiEntry& o, int k) {
+    const long double z = k / 64.0L, P = 0.5L * erfcl(-z * sqrtl(0.5L));
+    const long double l = expl(-0.5L * z * z) / (sqrtl(2.0L * 3.14159265358979323846264338327950288L) * P);
+    long double h0 = 1.0L, h1 = z, c = l;                    // He_{n-1}, He_n; l 2^-7n (-1)^(n-1) / n!
+    int e;
+    o.phi = to_q(frexpl(P, &e), 63);
+    o.e = e - 1;
+    o.pad = 0;
+    for (int n = 1; n <= 8; ++n) {
+        c = n == 1 ? l / 128.0L : -c / (128.0L * n);
+        if (n <= 4) o.c[n - 1] = to_q(c * h0, 62);
+        else o.b[n - 5] = (int)to_q(c * h0, 62);
+        const long double h2 = z * h1 - n * h0;
+        h0 = h1; h1 = h2;
+    }
+}
 inline void make_norm_tab(NormTab& t) {
+    for (int k = -PHI_SIDE; k <= PHI_SIDE; ++k) make_phi(t.phi[k + PHI_SIDE], k);
     for (int i = 0; i < 256; ++i) {
         const int inv = i == 255 ? 2048 : (int)lrint(4096.0 / (1.0 + (i + 0.5) / 256.0));
         t.lg[i] = LogEntry{inv == 2048 ? LN2_57 : to_q(-logl((long double)inv / 4096.0L), 57), inv, 0};

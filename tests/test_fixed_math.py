@@ -17,6 +17,10 @@ extern "C" void t_div(int n, const double* a, const double* b, double* q) { for 
 extern "C" void t_vg(int k, const double* ap, const double* n, const double* m, int* ok, double* s, double* kr, double* d) {
     for (int i = 0; i < k; ++i) { VgLog o; ok[i] = vg_log(ap[i], n[i], m[i], o); if (ok[i]) { s[i] = vg_s(o); vg_k(o, kr[i], d[i]); } }
 }
+extern "C" void t_cdf(int n, const double* x, double* y) {
+    static NormTab t; make_norm_tab(t);
+    for (int i = 0; i < n; ++i) y[i] = normal_cdf(x[i], t.phi);
+}
 extern "C" void t_normal(int k, const unsigned* c, double* y) {
     static NormTab t; make_norm_tab(t);
     for (int i = 0; i < k; ++i) { long long a, b; normal_pair(c[4*i], c[4*i+1], c[4*i+2], c[4*i+3], &t, a, b);
@@ -123,3 +127,18 @@ def test_normals_match_box_muller(lib):
     r = np.sqrt(-2.0 * np.log(u[0]))
     assert np.abs(y[:, 0] - r * np.cos(2 * np.pi * u[1])).max() < 5e-15
     assert np.abs(y[:, 1] - r * np.sin(2 * np.pi * u[1])).max() < 5e-15
+
+
+def test_normal_cdf_matches_erfc(lib):
+    """Against erfc in FP64 (2e-15 near -4, from the rounding of its argument);
+    both sides of the table's range, points midway between entries, tiny and
+    special values."""
+    import math
+    g = np.random.default_rng(4)
+    x = np.concatenate([g.standard_normal(20000), g.uniform(-5, 5, 20000), 2.0 ** g.uniform(-80, 0, 500) * g.choice([-1, 1], 500),
+                        np.arange(-520, 521) / 128.0, [0.0, -0.0, -30.0, 30.0, np.inf, -np.inf, np.nan, -4.0, 4.0]])
+    y = np.empty_like(x)
+    lib.t_cdf(len(x), dp(x), dp(y))
+    want = np.array([0.5 * math.erfc(-v / math.sqrt(2.0)) for v in x])
+    assert np.allclose(y, want, rtol=5e-15, atol=0, equal_nan=True)
+    assert y[x == 0].tolist() == [0.5, 0.5]
