@@ -208,15 +208,16 @@ constexpr long long CLUSTER_CELLS64 = 4096, CLUSTER_CELLS32 = 16384;
 // CTAs of a sample's cluster (0: one CTA per sample), with the plan of shared
 // memory made for it.  Only where the launch shape is free (rich_set_tuning 0),
 // for V-cycles, and when clusters for all samples are resident together.
-static int pick_cluster(const rich_ctx* ctx, const rich_problem_t* pb, int S, FParams& P, int* cluster) {
+using cluster_fn = int (*)(const FParams&, size_t smem, int n, int clusters, cudaStream_t, int* fit);
+static int pick_cluster(const rich_ctx* ctx, const rich_problem_t* pb, int S, FParams& P, cluster_fn call, int* cluster) {
     *cluster = 0;
     const long long cells = P.mixed ? CLUSTER_CELLS32 : CLUSTER_CELLS64;
-    if (ctx->tune_threads || P.gamma > 1 || (long long)pb->nx * pb->nz < cells || 2ll * S > ctx->sm_count) return 0;
+    if (S < 1 || ctx->tune_threads || P.gamma > 1 || (long long)pb->nx * pb->nz < cells || 2ll * S > ctx->sm_count) return 0;
     plan_smem(P, 512, cells);
     if (P.lx == 0) return 0;
     for (int n = std::min(8, ctx->sm_count / S); n >= 2; --n) {
         int fit = 0;
-        if (int e = fused_cluster(P, fused_smem(P), n, S, nullptr, &fit)) return e;
+        if (int e = call(P, fused_smem(P), n, S, nullptr, &fit)) return e;
         if (fit >= S) { *cluster = n; return 0; }
     }
     return 0;
@@ -236,7 +237,7 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     if (int e = fused_setup(pb, S, P)) return e;
     // a cluster of CTAs per sample where they all fit at once (grid: the clusters)
     int occ = 1, cluster = 0, grid = S;
-    if (int e = pick_cluster(ctx, pb, S, P, &cluster)) return e;
+    if (int e = pick_cluster(ctx, pb, S, P, fused_cluster, &cluster)) return e;
     if (cluster == 0) plan_smem(P, nt);
     if (soil) {
         P.n_in = soil->n; P.ts_in = soil->theta_s; P.tr_in = soil->theta_r;
@@ -287,17 +288,22 @@ int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const dou
     FParams P;
     if (ckpt_every < 1 || pb->closure != RICH_GARDNER) return RICH_ERR_INVALID;
     size_t smem = 0;
-    int grid = 0;
+    int grid = 0, cluster = 0;
     for (bool keep : {true, false}) {
         if (int e = fused_setup(pb, S, P, ckpt_every, keep)) return e;
-        plan_smem(P, 512);
+        // (the GMRES option keeps its small system in one CTA)
+        cluster = 0;
+        if (adj_method != 2)
+            if (int e = pick_cluster(ctx, pb, S, P, P.mixed ? rich_adjoint_cluster32 : rich_adjoint_cluster64, &cluster))
+                return e;
+        if (cluster == 0) plan_smem(P, 512);
         smem = fused_smem(P);
         int occ = 0;
         const void* kern = P.mixed ? rich_adjoint_kernel32(P.gamma > 1) : rich_adjoint_kernel64(P.gamma > 1);
         if (int e = allow_dyn_smem(kern, smem)) return e;
         RICH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 512, smem));
         occ = std::max(occ, 1);
-        grid = std::max(1, std::min(S, ctx->sm_count * occ));
+        grid = cluster ? S : std::max(1, std::min(S, ctx->sm_count * occ));
         if (keep && (size_t)grid * pb->nsteps * pb->nx * pb->nz * 8 > KEEP_STATES_BYTES) continue;
         const size_t need = (size_t)grid * (size_t)P.slot_bytes + 256;
         if (ctx->fused_bytes >= need) break;
@@ -320,7 +326,10 @@ int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const dou
     RICH_CUDA(cudaMemsetAsync(P.queue, 0, sizeof(int), st));
     rich_count_launch();
     rich_prof_begin(ctx, st);
-    if (P.mixed) rich_adjoint_launch32(P, grid, smem, st);
+    if (cluster) {
+        const auto call = P.mixed ? rich_adjoint_cluster32 : rich_adjoint_cluster64;
+        if (int e = call(P, smem, cluster, grid, st, nullptr)) return e;
+    } else if (P.mixed) rich_adjoint_launch32(P, grid, smem, st);
     else rich_adjoint_launch64(P, grid, smem, st);
     rich_prof_end(ctx, st, 0.0, 0.0);
     RICH_CUDA(cudaGetLastError());

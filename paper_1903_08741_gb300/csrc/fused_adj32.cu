@@ -14,4 +14,8 @@ void rich_adjoint_launch32(const FParams& P, int grid, size_t smem, cudaStream_t
     else k_adjoint<float, false><<<grid, 512, smem, st>>>(P);
 }
 
+int rich_adjoint_cluster32(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
+    return cluster_call(k_adjoint_cluster<float>, P, smem, n, clusters, st, fit);
+}
+
 }  // namespace rich_fused

@@ -13,7 +13,7 @@ void rich_launch_g32(const FParams& P, int grid, size_t smem, int nt, cudaStream
 }
 
 int rich_cluster_g32(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
-    return cluster_call<float, 0>(P, smem, n, clusters, st, fit);
+    return cluster_call(k_fused_cluster<float, 0>, P, smem, n, clusters, st, fit);
 }
 
 }  // namespace rich_fused

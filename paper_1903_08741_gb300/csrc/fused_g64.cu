@@ -13,7 +13,7 @@ void rich_launch_g64(const FParams& P, int grid, size_t smem, int nt, cudaStream
 }
 
 int rich_cluster_g64(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
-    return cluster_call<double, 0>(P, smem, n, clusters, st, fit);
+    return cluster_call(k_fused_cluster<double, 0>, P, smem, n, clusters, st, fit);
 }
 
 }  // namespace rich_fused

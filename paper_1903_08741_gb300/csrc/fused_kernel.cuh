@@ -145,6 +145,8 @@ int rich_cluster_vg32(const FParams& P, size_t smem, int n, int clusters, cudaSt
 // kernel's address (occupancy queries) and its launch with 512 threads
 const void* rich_adjoint_kernel64(bool wcycle);
 const void* rich_adjoint_kernel32(bool wcycle);
+int rich_adjoint_cluster64(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit);
+int rich_adjoint_cluster32(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit);
 void rich_adjoint_launch64(const FParams& P, int grid, size_t smem, cudaStream_t st);
 void rich_adjoint_launch32(const FParams& P, int grid, size_t smem, cudaStream_t st);
 
@@ -928,6 +930,21 @@ struct Cta {
         }
         return v;
     }
+    // sum over the group in a fixed order, returned to every thread
+    __device__ __forceinline__ double gsum(double v) {
+        v = block_sum(v, reinterpret_cast<double*>(red));
+        if constexpr (CLU) {
+            auto c = GClu::c();
+            const int n = (int)c.num_blocks();
+            if ((int)threadIdx.x < n)
+                *c.map_shared_rank(&cred[cpar][c.block_rank()], threadIdx.x) = (unsigned long long)__double_as_longlong(v);
+            c.sync();
+            v = 0.0;
+            for (int k = 0; k < n; ++k) v += __longlong_as_double((long long)cred[cpar][k]);
+            cpar ^= 1;
+        }
+        return v;
+    }
     // a level's threads in the set-up loops: a cluster's levels beyond lx belong
     // to its first CTA (their arrays may be in its shared memory)
     __device__ __forceinline__ bool mine(int l) const { return !CLU || l <= P.lx || tid < (int)blockDim.x; }
@@ -1308,7 +1325,7 @@ struct Cta {
             else d += F.Tbb[i];
             dE[q] = e; dW[q] = w; dN[q] = n; dS[q] = s; dg[q] = d;
         }
-        __syncthreads();
+        G0::sync();
     }
 
     __device__ __forceinline__ double jt_apply(const double* dE, const double* dW, const double* dN,
@@ -1335,7 +1352,7 @@ struct Cta {
             M0.f[sq] = SC ? v : (TM)r[q];
             start_cell(M0, q - j * nx, j, v);
         }
-        __syncthreads();
+        G0::sync();
         for (int k = 0; k < ninner; ++k) {
             if constexpr (SC) mgcycle(r, k == 0);
             else mgcycle(nullptr, k == 0);
@@ -1355,7 +1372,7 @@ struct Cta {
             unsigned long long b = abs_bits(rhs[q]);
             m = b > m ? b : m;
         }
-        const unsigned long long b0 = block_max(m, red);
+        const unsigned long long b0 = gmax(m);
         const double target = P.adj_tol * __longlong_as_double((long long)b0);
         if (b0 == 0) return 0;
         for (int it = 1; it <= P.adj_maxit; ++it) {
@@ -1364,7 +1381,7 @@ struct Cta {
                 const int j = fdiv(q, nx, L64[0].mnx);
                 lam[q] += (double)dp_at(M0, q - j * nx, j);
             }
-            __syncthreads();
+            G0::sync();
             unsigned long long mm = 0;
             for (int q = tid; q < nc; q += nt) {
                 double v = rhs[q] - jt_apply(dE, dW, dN, dS, dg, lam, q);
@@ -1372,7 +1389,7 @@ struct Cta {
                 unsigned long long b = abs_bits(v);
                 mm = b > mm ? b : mm;
             }
-            const unsigned long long rb = block_max(mm, red);
+            const unsigned long long rb = gmax(mm);
             if (rb > INF_BITS - 1) return P.adj_maxit + 1;
             if (__longlong_as_double((long long)rb) <= target) return it;
         }
@@ -1387,14 +1404,14 @@ struct Cta {
             const int j = fdiv(q, nx, L64[0].mnx);
             out[q] = (double)dp_at(LM[0], q - j * nx, j);
         }
-        __syncthreads();
+        G0::sync();
     }
 
     // y = J^T x over all cells, then the CTA synchronises
     __device__ void jt_vec(const double* dE, const double* dW, const double* dN, const double* dS,
                            const double* dg, const double* x, double* y) {
         for (int q = tid; q < nc; q += nt) y[q] = jt_apply(dE, dW, dN, dS, dg, x, q);
-        __syncthreads();
+        G0::sync();
     }
 
     // J^T lam = rhs by BiCGStab (van der Vorst 1992) right-preconditioned with
@@ -1406,14 +1423,13 @@ struct Cta {
     __device__ int adj_solve_bicgstab(const double* dE, const double* dW, const double* dN, const double* dS,
                                       const double* dg, const double* rhs, double* lam, double* r, double* rh,
                                       double* pk, double* v, double* t, double* ph, double* sh) {
-        double* redd = reinterpret_cast<double*>(red);
         unsigned long long m = 0;
         for (int q = tid; q < nc; q += nt) {
             lam[q] = 0.0;
             unsigned long long b = abs_bits(rhs[q]);
             m = b > m ? b : m;
         }
-        const unsigned long long b0 = block_max(m, red);
+        const unsigned long long b0 = gmax(m);
         if (b0 == 0) return 0;
         const double target = P.adj_tol * __longlong_as_double((long long)b0);
         int apps = 0;
@@ -1428,7 +1444,7 @@ struct Cta {
                     unsigned long long b = abs_bits(rv);
                     rm = b > rm ? b : rm;
                 }
-                const unsigned long long rb = block_max(rm, red);
+                const unsigned long long rb = gmax(rm);
                 if (rb > INF_BITS - 1) break;
                 if (__longlong_as_double((long long)rb) <= target) return apps;
                 rho = alpha = omega = 1.0;
@@ -1437,16 +1453,16 @@ struct Cta {
             }
             double s1 = 0.0;
             for (int q = tid; q < nc; q += nt) s1 += rh[q] * r[q];
-            const double rho_new = block_sum(s1, redd);
+            const double rho_new = gsum(s1);
             if (!(fabs(rho_new) > 0.0) || !isfinite(rho_new)) { restart = true; if (!isfinite(rho_new)) break; continue; }
             const double beta = (rho_new / rho) * (alpha / omega);
             for (int q = tid; q < nc; q += nt) pk[q] = r[q] + beta * (pk[q] - omega * v[q]);
-            __syncthreads();
+            G0::sync();
             precond(pk, ph); ++apps;
             jt_vec(dE, dW, dN, dS, dg, ph, v);
             double s2 = 0.0;
             for (int q = tid; q < nc; q += nt) s2 += rh[q] * v[q];
-            const double den = block_sum(s2, redd);
+            const double den = gsum(s2);
             if (!(fabs(den) > 0.0) || !isfinite(den)) { restart = true; if (!isfinite(den)) break; continue; }
             alpha = rho_new / den;
             unsigned long long sm = 0;
@@ -1456,11 +1472,11 @@ struct Cta {
                 unsigned long long b = abs_bits(sv);
                 sm = b > sm ? b : sm;
             }
-            const unsigned long long sb = block_max(sm, red);
+            const unsigned long long sb = gmax(sm);
             if (sb > INF_BITS - 1) break;
             if (__longlong_as_double((long long)sb) <= target) {
                 for (int q = tid; q < nc; q += nt) lam[q] += alpha * ph[q];
-                __syncthreads();
+                G0::sync();
                 if (true_resid_ok(dE, dW, dN, dS, dg, rhs, lam, target)) return apps;
                 restart = true;
                 continue;
@@ -1469,8 +1485,8 @@ struct Cta {
             jt_vec(dE, dW, dN, dS, dg, sh, t);
             double s3 = 0.0, s4 = 0.0;
             for (int q = tid; q < nc; q += nt) { s3 += t[q] * r[q]; s4 += t[q] * t[q]; }
-            const double ts = block_sum(s3, redd);
-            const double tt = block_sum(s4, redd);
+            const double ts = gsum(s3);
+            const double tt = gsum(s4);
             omega = tt > 0.0 ? ts / tt : 0.0;
             unsigned long long rm = 0;
             for (int q = tid; q < nc; q += nt) {
@@ -1480,7 +1496,7 @@ struct Cta {
                 unsigned long long b = abs_bits(rv);
                 rm = b > rm ? b : rm;
             }
-            const unsigned long long rb = block_max(rm, red);
+            const unsigned long long rb = gmax(rm);
             if (rb > INF_BITS - 1) break;
             if (__longlong_as_double((long long)rb) <= target) {
                 if (true_resid_ok(dE, dW, dN, dS, dg, rhs, lam, target)) return apps;
@@ -1498,7 +1514,7 @@ struct Cta {
     // rotations; each cycle ends with the update lam += Z y and the TRUE
     // residual ||rhs - J^T lam||_inf <= adj_tol ||rhs||_inf decides.  The
     // Hessenberg matrix and rotations are computed by every thread from the
-    // same block sums (uniform control flow).  Returns the number of
+    // same block sums (uniform control flow).  One CTA only (not a cluster).  Returns the number of
     // preconditioner applications (adj_maxit + 1 when not converged).
     __device__ int adj_solve_gmres(const double* dE, const double* dW, const double* dN, const double* dS,
                                    const double* dg, const double* rhs, double* lam, double* kry) {
@@ -1609,7 +1625,7 @@ struct Cta {
             unsigned long long b = abs_bits(rhs[q] - jt_apply(dE, dW, dN, dS, dg, lam, q));
             m = b > m ? b : m;
         }
-        const unsigned long long rb = block_max(m, red);
+        const unsigned long long rb = gmax(m);
         return rb <= INF_BITS - 1 && __longlong_as_double((long long)rb) <= target;
     }
 
@@ -1634,7 +1650,7 @@ struct Cta {
             else v -= (P.p_bot - pc - h / 2.0) * F.Tbb[i] * lc;
             g[q] -= v;
         }
-        __syncthreads();
+        G0::sync();
     }
 };
 
@@ -1799,8 +1815,8 @@ void launch_shapes(const FParams& P, int grid, size_t smem, int nt, cudaStream_t
 
 // clusters of n CTAs: fit != null asks how many the GPU holds at a time, else
 // `clusters` of them are launched
-template <typename TM, int CL>
-int cluster_call(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
+inline int cluster_call(void (*kernel)(FParams), const FParams& P, size_t smem, int n, int clusters, cudaStream_t st,
+                        int* fit) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
@@ -1808,11 +1824,11 @@ int cluster_call(const FParams& P, size_t smem, int n, int clusters, cudaStream_
     cfg.gridDim = dim3((unsigned)(clusters * n)); cfg.blockDim = dim3(CLUSTER_THREADS);
     cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = at; cfg.numAttrs = 1;
     if (fit) {
-        if (int e = allow_dyn_smem((const void*)k_fused_cluster<TM, CL>, smem)) return e;
-        RICH_CUDA(cudaOccupancyMaxActiveClusters(fit, k_fused_cluster<TM, CL>, &cfg));
+        if (int e = allow_dyn_smem((const void*)kernel, smem)) return e;
+        RICH_CUDA(cudaOccupancyMaxActiveClusters(fit, kernel, &cfg));
         return 0;
     }
-    RICH_CUDA(cudaLaunchKernelEx(&cfg, k_fused_cluster<TM, CL>, P));
+    RICH_CUDA(cudaLaunchKernelEx(&cfg, kernel, P));
     return 0;
 }
 }  // namespace

@@ -13,7 +13,7 @@ void rich_launch_vg64(const FParams& P, int grid, size_t smem, int nt, cudaStrea
 }
 
 int rich_cluster_vg64(const FParams& P, size_t smem, int n, int clusters, cudaStream_t st, int* fit) {
-    return cluster_call<double, 1>(P, smem, n, clusters, st, fit);
+    return cluster_call(k_fused_cluster<double, 1>, P, smem, n, clusters, st, fit);
 }
 
 }  // namespace rich_fused

@@ -48,3 +48,28 @@ def test_cluster_matches_one_cta_van_genuchten(R, precision):
     finally:
         R.set_tuning(0, 0)
     assert torch.equal(a[2], b[2]) and torch.equal(a[1].nan_to_num(7.0), b[1].nan_to_num(7.0))
+
+
+@pytest.mark.parametrize("method,n,S,precision", [(0, 64, 2, 0), (1, 64, 50, 0), (1, 128, 3, 1), (2, 64, 3, 0)])
+def test_adjoint_cluster_matches_one_cta(R, method, n, S, precision):
+    """Same forward bits; the J^T solves differ by the order of their sums, within
+    their 1e-11 residual target times the operators' condition: 1e-8."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    basis = torch.randn((4, n, n), dtype=torch.float64, device="cuda", generator=g) * 0.05
+    xi = torch.randn((S, 4), dtype=torch.float64, device="cuda", generator=g)
+    al = torch.full((S, n, n), 0.7, dtype=torch.float64, device="cuda")
+    pb = R.Problem(nx=n, nz=n, nsteps=3, dt=0.01, precision=precision)
+    out = []
+    try:
+        assert R.lib().rich_set_adjoint_method(R.context(0), method) == 0
+        for nt in (0, 512):
+            R.set_tuning(nt, 0)
+            out.append(R.solve_batch_adjoint(pb, basis, xi, al))
+    finally:
+        R.set_tuning(0, 0)
+        R.lib().rich_set_adjoint_method(R.context(0), 1)
+    a, b = out
+    assert torch.equal(a[0], b[0]) and torch.isfinite(a[1]).all()
+    assert (a[1] - b[1]).abs().max() <= 1e-8 * b[1].abs().max()
+    if method == 2:
+        assert torch.equal(a[1], b[1])
