@@ -14,7 +14,7 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Dynamic shared memory of a CTA (no device work): the coarsest level's
 // factored matrix; then the arrays that the cycles read on the small coarse levels
-// that warp 0 runs alone (levels l >= 1 with at most WARP_CELLS cells: the
+// (levels l >= 1 with at most WARP_CELLS cells: the
 // multigrid arrays, and for FP64 the coarsest level's faces and diagonal,
 // from which the matrix is assembled); then the corrections dp of as many of the other levels
 // (coarsest first) as fit the budget of the launch shape (one 1024-thread CTA
@@ -24,6 +24,13 @@ size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 // stay on chip; levels that do not fit keep dp in the slot.  Results do not
 // depend on where an array lives.
 constexpr int WARP_CELLS = 256;
+// Warp 0 alone runs the on-chip levels, in FP64 only those of at most 64 cells: it
+// reaches a quarter of the SM's FP64 pipe, where a half-sweep of a 16^2 level takes
+// 1024 clocks against 256 on four warps, more than the barrier it saves (ms with
+// 256 / 64 / 16 cells: 32^2 x 64 117 / 104 / 104, 64^2 x 1 103 / 96 / 97, 32^2 x 608
+// 82 / 71 / 75, 64^2 x 48 adjoint 146 / 137 / 138, cost map 188 / 184 / 188, a
+// 16^2...64^2 MLMC estimate 707 / 666 / 686; full batches of large grids alike).
+constexpr int WARP_CELLS64 = 64;
 
 // A cluster (cells > 0) runs its levels of at least `cells` cells on all its CTAs
 // (lx of them): their corrections, and the next level's, stay in the slot.
@@ -43,12 +50,14 @@ static void plan_smem(FParams& P, int nt, long long cells = 0) {
     // small levels below the finest run on warp 0 with their arrays on chip;
     // a one-warp CTA (32 threads, 32 CTAs per SM) runs every level itself and
     // keeps them in its slot: on-chip copies would cost it its occupancy
-    P.lw = P.nlev;
+    int ls = P.nlev;                          // first level with its arrays on chip
     for (int l = 1; l < P.nlev && nt > 32; ++l)
-        if ((size_t)P.nx[l] * P.nz[l] <= (size_t)WARP_CELLS) { P.lw = l; break; }
+        if ((size_t)P.nx[l] * P.nz[l] <= (size_t)WARP_CELLS) { ls = l; break; }
+    P.lw = ls;
+    while (!P.mixed && P.lw < P.nlev && P.nx[P.lw] * P.nz[P.lw] > WARP_CELLS64) ++P.lw;
     P.lx = 0;
-    while (cells > 0 && P.lx < std::min(P.lw, P.nlev - 1) - 1 && (long long)P.nx[P.lx] * P.nz[P.lx] >= cells) ++P.lx;
-    for (int l = P.lw; l < P.nlev; ++l) {
+    while (cells > 0 && P.lx < std::min(ls, P.nlev - 1) - 1 && (long long)P.nx[P.lx] * P.nz[P.lx] >= cells) ++P.lx;
+    for (int l = ls; l < P.nlev; ++l) {
         const size_t nc = (size_t)P.nx[l] * P.nz[l];
         if (!P.mixed) {
             for (int k = 0; k < N64; ++k) {
@@ -63,7 +72,7 @@ static void plan_smem(FParams& P, int nt, long long cells = 0) {
             off = al16(off + nc * w);
         }
     }
-    for (int l = P.lw - 1; l >= (P.lx > 0 ? P.lx + 1 : 0); --l) {
+    for (int l = ls - 1; l >= (P.lx > 0 ? P.lx + 1 : 0); --l) {
         const size_t bytes = al16((size_t)P.nx[l] * P.nz[l] * w);
         if (off + bytes > budget) break;
         P.osm[l] = (long long)off;

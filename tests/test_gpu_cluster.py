@@ -73,3 +73,24 @@ def test_adjoint_cluster_matches_one_cta(R, method, n, S, precision):
     assert (a[1] - b[1]).abs().max() <= 1e-8 * b[1].abs().max()
     if method == 2:
         assert torch.equal(a[1], b[1])
+
+
+def test_cluster_launch_is_captured(R):
+    """A cluster launch inside a CUDA graph replays to the direct call's bits."""
+    from tests.inputs import smooth_random_fields
+    n, S = 64, 3
+    lk, al = (torch.from_numpy(v).cuda() for v in smooth_random_fields(n, n, S, 2))
+    pb = R.Problem(nx=n, nz=n, nsteps=2, dt=0.01)
+    q, st = torch.empty(S, dtype=torch.float64, device="cuda"), torch.empty(S, dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        R.solve_batch_async(pb, lk, al, q, st)                      # set-up outside the capture
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            R.solve_batch_async(pb, lk, al, q, st)
+    q.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    want = R.solve_batch(pb, lk, al)
+    assert torch.equal(q.nan_to_num(7.0), want[0].nan_to_num(7.0)) and torch.equal(st, want[2])
