@@ -265,9 +265,9 @@ __device__ __forceinline__ Nb nb_half(int col, int c, int i, int hx, int H) {
 template <typename T> struct Scaled { static constexpr bool value = sizeof(T) == 8; };
 
 // Thread groups that run a level's loops: the whole CTA (barrier
-// __syncthreads), or warp 0 alone (barrier __syncwarp) on the small coarse
-// levels, whose few hundred cells do not pay for CTA-wide barriers; those
-// levels keep every array in shared memory.  Each level function ends with
+// __syncthreads), warp 0 alone (barrier __syncwarp) on the smallest coarse
+// levels, whose cells do not pay for CTA-wide barriers and which keep every
+// array in shared memory, or a cluster of CTAs.  Each level function ends with
 // its group synchronised.
 struct GCta {
     static __device__ __forceinline__ int rank() { return threadIdx.x; }
