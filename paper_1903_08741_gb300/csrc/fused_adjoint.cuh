@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(CLUSTER_THREADS, 1)
 k_adjoint_cluster(const FParams P) {
     extern __shared__ unsigned char smraw[];
     __shared__ unsigned long long red[33];
-    __shared__ unsigned long long cred[2][8];
+    __shared__ unsigned long long cred[2][CLUSTER_THREADS / 32];
     __shared__ int s_sample;
     __shared__ Lv64 L64[MAXL];
     __shared__ Lv<TM> LM[MAXL];

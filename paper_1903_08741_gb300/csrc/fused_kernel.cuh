@@ -281,6 +281,7 @@ struct GWarp {
 };
 // all CTAs of a thread-block cluster (one sample): the barrier orders their
 // global and shared accesses
+constexpr int CLUSTER_THREADS = 512;
 struct GClu {
     static __device__ __forceinline__ cooperative_groups::cluster_group c() { return cooperative_groups::this_cluster(); }
     static __device__ __forceinline__ int rank() { return (int)(c().block_rank() * blockDim.x + threadIdx.x); }
@@ -889,7 +890,8 @@ struct Cta {
     Lv<TM>* LM;
     TM* Amat;
     unsigned long long* red;
-    unsigned long long (*cred)[8] = nullptr;   // cluster: the CTAs' maxima, two sets used in turn
+    // cluster: the CTAs' maxima, or the warps' sums (gdot); two sets used in turn
+    unsigned long long (*cred)[CLUSTER_THREADS / 32] = nullptr;
     int cpar = 0;
     double *f64, *dp64, *p, *thold, *Ks, *aa, *K, *th;
     double *nn, *mm, *trc, *tsc;          // closure 1: per-cell n, m, theta_r, theta_s
@@ -930,20 +932,36 @@ struct Cta {
         }
         return v;
     }
-    // sum over the group in a fixed order, returned to every thread
-    __device__ __forceinline__ double gsum(double v) {
-        v = block_sum(v, reinterpret_cast<double*>(red));
+    // sum of a b over the cells, returned to every thread: one CTA's 512 chains
+    // (cell q in chain q mod 512), its warps' trees and the tree over the warps, on
+    // any group, so that a sample's sums do not depend on how many CTAs, and with
+    // them how many other samples, the call gives it.  A cluster deals the 16
+    // warps' chains out to its CTAs; a and b are complete (a barrier lies behind).
+    __device__ __forceinline__ double gdot(const double* a, const double* b) {
+        double s = 0.0;
         if constexpr (CLU) {
+            constexpr int NW = CLUSTER_THREADS / 32;
             auto c = GClu::c();
-            const int n = (int)c.num_blocks();
-            if ((int)threadIdx.x < n)
-                *c.map_shared_rank(&cred[cpar][c.block_rank()], threadIdx.x) = (unsigned long long)__double_as_longlong(v);
+            const int n = (int)c.num_blocks(), lane = threadIdx.x & 31;
+            const int w = (int)(threadIdx.x >> 5) * n + (int)c.block_rank();
+            if (w < NW) {
+#pragma unroll 8
+                for (int q = 32 * w + lane; q < nc; q += CLUSTER_THREADS) s = fma(a[q], b[q], s);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane < n)
+                    *c.map_shared_rank(&cred[cpar][w], lane) = (unsigned long long)__double_as_longlong(s);
+            }
             c.sync();
-            v = 0.0;
-            for (int k = 0; k < n; ++k) v += __longlong_as_double((long long)cred[cpar][k]);
+            s = lane < NW ? __longlong_as_double((long long)cred[cpar][lane]) : 0.0;
             cpar ^= 1;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            return s;
+        } else {
+            for (int q = tid; q < nc; q += nt) s = fma(a[q], b[q], s);
+            return block_sum(s, reinterpret_cast<double*>(red));
         }
-        return v;
     }
     // a level's threads in the set-up loops: a cluster's levels beyond lx belong
     // to its first CTA (their arrays may be in its shared memory)
@@ -1451,18 +1469,14 @@ struct Cta {
                 restart = false;
                 if (apps > 0) ++apps;               // a restart counts as one application
             }
-            double s1 = 0.0;
-            for (int q = tid; q < nc; q += nt) s1 += rh[q] * r[q];
-            const double rho_new = gsum(s1);
+            const double rho_new = gdot(rh, r);
             if (!(fabs(rho_new) > 0.0) || !isfinite(rho_new)) { restart = true; if (!isfinite(rho_new)) break; continue; }
             const double beta = (rho_new / rho) * (alpha / omega);
             for (int q = tid; q < nc; q += nt) pk[q] = r[q] + beta * (pk[q] - omega * v[q]);
             G0::sync();
             precond(pk, ph); ++apps;
             jt_vec(dE, dW, dN, dS, dg, ph, v);
-            double s2 = 0.0;
-            for (int q = tid; q < nc; q += nt) s2 += rh[q] * v[q];
-            const double den = gsum(s2);
+            const double den = gdot(rh, v);
             if (!(fabs(den) > 0.0) || !isfinite(den)) { restart = true; if (!isfinite(den)) break; continue; }
             alpha = rho_new / den;
             unsigned long long sm = 0;
@@ -1483,10 +1497,8 @@ struct Cta {
             }
             precond(r, sh); ++apps;
             jt_vec(dE, dW, dN, dS, dg, sh, t);
-            double s3 = 0.0, s4 = 0.0;
-            for (int q = tid; q < nc; q += nt) { s3 += t[q] * r[q]; s4 += t[q] * t[q]; }
-            const double ts = gsum(s3);
-            const double tt = gsum(s4);
+            const double ts = gdot(t, r);
+            const double tt = gdot(t, t);
             omega = tt > 0.0 ? ts / tt : 0.0;
             unsigned long long rm = 0;
             for (int q = tid; q < nc; q += nt) {
@@ -1739,13 +1751,12 @@ k_fused(const FParams P) {
 // with the reads that follow it) after each.  Fine levels run on all CTAs, their
 // arrays in the slot; the first CTA runs the rest (vcycle).  256^2 x 24 samples,
 // mixed: 247 -> 86 ms; one 64^2 sample, FP64: 146 -> 104 ms.
-constexpr int CLUSTER_THREADS = 512;
 template <typename TM, int CL>
 __global__ void __launch_bounds__(CLUSTER_THREADS, 1)
 k_fused_cluster(const FParams P) {
     extern __shared__ unsigned char smraw[];
     __shared__ unsigned long long red[33];
-    __shared__ unsigned long long cred[2][8];
+    __shared__ unsigned long long cred[2][CLUSTER_THREADS / 32];
     __shared__ int s_sample;
     __shared__ Lv64 L64[MAXL];
     __shared__ Lv<TM> LM[MAXL];
