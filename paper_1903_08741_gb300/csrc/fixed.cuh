@@ -257,15 +257,17 @@ FXD unsigned long long exp_core(int k, long long r, int& n) {
     return v << 1;
 }
 
-// v 2^n (v in Q62) rounded to FP64; the result is normal
-FX double fx_to_double(unsigned long long v, int n) {
-    const unsigned long long m = (v + 512) >> 10;            // 2^52 <= m <= 2^53
-    const unsigned long long b = m + ((unsigned long long)(n + 1022) << 52);
+FX double bits_double(unsigned long long b) {
 #ifdef __CUDA_ARCH__
     return __longlong_as_double((long long)b);
 #else
     double d; memcpy(&d, &b, 8); return d;
 #endif
+}
+// v 2^n (v in Q62) rounded to FP64; the result is normal
+FX double fx_to_double(unsigned long long v, int n) {
+    const unsigned long long m = (v + 512) >> 10;            // 2^52 <= m <= 2^53
+    return bits_double(m + ((unsigned long long)(n + 1022) << 52));
 }
 FX unsigned long long double_bits(double x) {
 #ifdef __CUDA_ARCH__
@@ -294,16 +296,19 @@ FXD double fx_exp(double x) {
     return fx_to_double(v, n);
 }
 
-// a / b to 0.51 units in the last place where both are positive and normal and
-// the quotient is well inside the normal range (all else: the FP64 division,
-// which holds its pipe for about 9 multiply-adds, two to four of them a cell and
-// Picard iteration: 608 samples on 128^2 are 4.8 % faster in mixed precision and
-// 2.7 % in FP64): a 23-bit reciprocal of b and its third-order correction
+// a / b, correctly rounded, where both are positive and normal and the quotient is
+// well inside the normal range (all else: the FP64 division, which holds its pipe
+// for about 9 multiply-adds, two to four of them a cell and Picard iteration).  A
+// 23-bit reciprocal of b and its third-order correction give the quotient to within
+// a unit of its last place, and the exact remainder against half of b decides that
+// unit (no quotient of two 53-bit numbers lies midway).  Against the FP64 division,
+// same bits: 608 samples on 128^2, two steps, in mixed precision 290 -> 276 ms, in
+// FP64 542 -> 532 (runs 4 % apart), 64 samples on 32^2, ten steps, 98.9 -> 98.1.
 FX double fx_div(double a, double b) {
     const unsigned long long ba = double_bits(a), bb = double_bits(b), one = 1ull << 52;
     const int ea = (int)(ba >> 52), eb = (int)(bb >> 52), ex = ea - eb + 1023;
     if ((unsigned)(ea - 1) >= 2046u || (unsigned)(eb - 1) >= 2046u || ex < 8 || ex > 2038) return a / b;
-    const unsigned long long B = (bb | one) << 11;           // [2^63, 2^64): b's mantissa in Q63
+    const unsigned long long ma = (ba & (one - 1)) | one, mb = (bb & (one - 1)) | one, B = mb << 11;   // (B in Q63)
     const unsigned int fb = 0x3F800000u | ((unsigned int)(B >> 40) & 0x7FFFFFu);
 #ifdef __CUDA_ARCH__
     const unsigned int fy = __float_as_uint(__frcp_rn(__uint_as_float(fb)));
@@ -317,10 +322,13 @@ FX double fx_div(double a, double b) {
     const long long dh = d >> 16;
     const long long c = d + ((dh * dh) >> 30);
     const long long y = ((long long)Y << 31) + rmul(c, (long long)Y << 31);
-    unsigned long long q = (unsigned long long)rmul((long long)((ba & (one - 1)) | one) << 9, y);   // a/b in Q61
-    int n = ex - 1023;
-    if (!(q >> 61)) { q <<= 1; --n; }
-    return fx_to_double(q << 1, n);
+    const long long q = rmul((long long)ma << 9, y);         // ma / mb in Q61, good to 2^-58
+    // 53 bits of it, exactly s fraction bits, and their remainder, modulo 2^64
+    const int s = ma < mb ? 53 : 52;
+    unsigned long long m = (unsigned long long)((q + (1ll << (60 - s))) >> (61 - s));
+    const long long rem = (long long)((ma << s) - m * mb);
+    m += (unsigned long long)((long long)(2 * rem > (long long)mb) - (long long)(2 * rem < -(long long)mb));
+    return bits_double(m + ((unsigned long long)(ex - 1 + 52 - s) << 52));
 }
 
 // e^(y 2^-F), |y 2^-F| < 512, as v 2^n
