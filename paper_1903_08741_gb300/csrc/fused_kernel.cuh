@@ -973,6 +973,14 @@ struct Cta {
         else if (tid < (int)blockDim.x) __syncthreads();
     }
 
+    // the assembly's quotients (the same bits either way): with the van Genuchten
+    // closure the integer pipes are the busier ones and the FP64 division is faster
+    // (the cost map, 4096 samples of 32^2: 172 -> 168 ms), with Gardner's it is not (fixed.cuh)
+    static __device__ __forceinline__ double quot(double a, double b) {
+        if constexpr (CL == 0) return rich_fx::fx_div(a, b);
+        else return a / b;
+    }
+
     // conductivity of cell q's soil at head pp (Dirichlet faces, QoI)
     __device__ __forceinline__ double k_at(int q, double pp) const {
         if constexpr (CL == 0) {
@@ -1084,9 +1092,9 @@ struct Cta {
         for (int q = tid; q < nc; q += nt) {
             int j = fdiv(q, nx, F.mnx), i = q - j * nx;
             double kp = K[q];
-            if (i < nx - 1) { double ke = K[q + 1]; F.Tx[q] = rich_fx::fx_div(t2h * kp * ke, kp + ke); }
+            if (i < nx - 1) { double ke = K[q + 1]; F.Tx[q] = quot(t2h * kp * ke, kp + ke); }
             else F.Tx[q] = 0.0;
-            if (j < nz - 1) { double kn = K[q + nx]; F.Tz[q] = rich_fx::fx_div(t2h * kp * kn, kp + kn); }
+            if (j < nz - 1) { double kn = K[q + nx]; F.Tz[q] = quot(t2h * kp * kn, kp + kn); }
             else F.Tz[q] = 0.0;
         }
         G0::sync();
@@ -1107,7 +1115,7 @@ struct Cta {
             f64[q] = -R;
             const int sq = sidx(M0, i, j);
             if constexpr (SC) {
-                double inv = rich_fx::fx_div(1.0, d);
+                double inv = quot(1.0, d);
                 M0.q[sq] = inv; M0.D[sq] = d;
                 M0.c0[sq] = te * inv; M0.c1[sq] = tw * inv; M0.c2[sq] = tn * inv; M0.c3[sq] = tsf * inv;
                 M0.f[sq] = -R * inv;
@@ -1145,7 +1153,7 @@ struct Cta {
                 if (SC && l == nlev - 1) Cl.D[c] = d;
                 const int sc = sidx(Ml, I, J);
                 if constexpr (SC) {
-                    double inv = rich_fx::fx_div(1.0, d);
+                    double inv = quot(1.0, d);
                     Ml.q[sc] = 0.25 * inv; Ml.D[sc] = d;
                     Ml.c0[sc] = te * inv; Ml.c1[sc] = tw * inv; Ml.c2[sc] = tn * inv; Ml.c3[sc] = tsf * inv;
                 } else {
