@@ -383,10 +383,12 @@ int rich_kl_fields(rich_ctx_t ctx, const double* kl_basis, int32_t n_kl, int32_t
  * rich_set_adjoint_method) preconditioned with CCMG V-cycles of the Picard
  * operator (FP32 V-cycles when pb->precision is RICH_MIXED) to a relative
  * residual of 1e-11.  Memory: the states of all steps are kept while those of
- * the resident samples fit in 4 GiB; else they are checkpointed every
- * ckpt_every steps and each segment is recomputed during the reverse sweep.
+ * the resident samples fit in the limit of rich_set_adjoint_memory (4 GiB) and
+ * on the device; else they are checkpointed every ckpt_every steps and each
+ * segment is recomputed during the reverse sweep (the same bits, about twice the
+ * time).  Kept states of more than 64 MiB are freed before the call returns.
  * dq_dlnKs [S][nz][nx] (device) may be NULL.  A J^T solve that stops at its
- * iteration limit sets RICH_MG_MAXIT.  Synchronous (returns when done). */
+ * iteration limit sets RICH_ADJ_MAXIT.  Synchronous (returns when done). */
 int rich_solve_batch_adjoint(rich_ctx_t ctx, const rich_problem_t* pb, int32_t nsamples,
                              const double* kl_basis, int32_t n_kl, const double* xi,
                              const double* alpha, double alpha_scale, int32_t ckpt_every,
@@ -411,6 +413,13 @@ int rich_set_adjoint_method(rich_ctx_t ctx, int32_t method);
  * not fully converged gradient are still returned).  Defaults 1e-11 and 400.
  * RICH_ERR_INVALID unless 0 < rel_tol < 1 and 1 <= max_applications <= 1e6. */
 int rich_set_adjoint_limits(rich_ctx_t ctx, double rel_tol, int32_t max_applications);
+
+/* Device memory that this context's adjoint calls may use to keep the states of
+ * every time step of their resident samples (default 4 GiB).  A call that would
+ * need more checkpoints them every ckpt_every steps; 0: every call does.  States
+ * kept from an earlier call beyond the new limit are freed.  RICH_ERR_INVALID if
+ * negative. */
+int rich_set_adjoint_memory(rich_ctx_t ctx, int64_t bytes);
 
 /* Allocation-free solve.  The paper has no counterpart: this entry point exists
  * for callers that cannot call cudaMalloc -- code embedded in a host framework

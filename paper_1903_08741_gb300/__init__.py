@@ -286,6 +286,7 @@ def lib():
         L.rich_measure_fp64.argtypes = [vp, C.POINTER(_Fp64Rates)]
         L.rich_set_adjoint_method.argtypes = [vp, i32]
         L.rich_set_adjoint_limits.argtypes = [vp, dbl, i32]
+        L.rich_set_adjoint_memory.argtypes = [vp, i64]
         _lib = L
     return _lib
 
@@ -298,7 +299,7 @@ def exported_symbols():
             "rich_kl_fields", "rich_solve_batch_adjoint", "rich_set_tuning", "rich_sample_fields_at",
             "rich_solve_batch_async", "rich_mlmc_adaptive", "rich_sample_soil", "rich_solve_soil",
             "rich_sample_soil_pair", "rich_sample_counters", "rich_measure_fp64",
-            "rich_set_adjoint_method", "rich_set_adjoint_limits"]
+            "rich_set_adjoint_method", "rich_set_adjoint_limits", "rich_set_adjoint_memory"]
 
 
 def _check(rc):
@@ -530,6 +531,12 @@ def set_adjoint_limits(rel_tol=1e-11, max_applications=400, device=0):
     """Stopping rule of the device's adjoint J^T solves: relative residual
     target and cap on preconditioner applications (then status ADJ_MAXIT)."""
     _check(lib().rich_set_adjoint_limits(context(device), float(rel_tol), int(max_applications)))
+
+
+def set_adjoint_memory(nbytes=4 << 30, device=0):
+    """Device memory that the device's adjoint solves may use to keep the states
+    of every step; beyond it (0: always) they checkpoint every ckpt_every steps."""
+    _check(lib().rich_set_adjoint_memory(context(device), int(nbytes)))
 
 
 def measure_fp64(device=0):

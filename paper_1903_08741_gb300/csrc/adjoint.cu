@@ -44,6 +44,12 @@ __global__ void k_kl_project(int nkl, int nc, const double* __restrict__ basis,
     if (threadIdx.x == 0) out[(size_t)s * nkl + j] = sm[0];
 }
 
+void drop_states(rich_ctx* c) {
+    if (c->adj_states) cudaFree(c->adj_states);
+    c->adj_states = nullptr;
+    c->adj_states_bytes = 0;
+}
+
 }  // namespace
 
 extern "C" int rich_kl_fields(rich_ctx_t ctx, const double* basis, int32_t n_kl, int32_t ncell,
@@ -78,6 +84,11 @@ extern "C" int rich_solve_batch_adjoint(rich_ctx_t ctx, const rich_problem_t* pb
     double* g = dq_dlnKs ? dq_dlnKs : lk + (size_t)nsamples * nc;
     if (int e = rich_kl_fields(ctx, kl_basis, n_kl, nc, xi, nsamples, lk, stream)) return e;
     if (int e = rich_samples_reserve(ctx, nsamples)) return e;
+    // whichever way the call ends (cudaFree waits for work in flight)
+    struct GiveBack {
+        rich_ctx* c;
+        ~GiveBack() { if (c->adj_states_bytes > ADJ_STATES_POOL) drop_states(c); }
+    } give_back{ctx};
     auto t0 = std::chrono::steady_clock::now();
     // adjoint linear solves to the context's relative residual (default 1e-11),
     // at most its cap of preconditioner applications (default 400)
@@ -115,6 +126,14 @@ extern "C" int rich_solve_batch_adjoint(rich_ctx_t ctx, const rich_problem_t* pb
 extern "C" int rich_set_adjoint_method(rich_ctx_t ctx, int32_t method) {
     if (!ctx || method < 0 || method > 2) return RICH_ERR_INVALID;
     ctx->adj_method = method;
+    return 0;
+}
+
+extern "C" int rich_set_adjoint_memory(rich_ctx_t ctx, int64_t bytes) {
+    if (!ctx || bytes < 0) return RICH_ERR_INVALID;
+    RICH_CUDA(cudaSetDevice(ctx->device));
+    ctx->adj_memory = (size_t)bytes;
+    if (ctx->adj_states_bytes > ctx->adj_memory) drop_states(ctx);
     return 0;
 }
 

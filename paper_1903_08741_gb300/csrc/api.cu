@@ -127,6 +127,7 @@ extern "C" void rich_destroy(rich_ctx_t ctx) {
     if (ctx->field_work) cudaFree(ctx->field_work);
     for (auto e : ctx->prof.ev) cudaEventDestroy(e);
     if (ctx->fused_scratch) cudaFree(ctx->fused_scratch);
+    if (ctx->adj_states) cudaFree(ctx->adj_states);
     delete ctx;
 }
 

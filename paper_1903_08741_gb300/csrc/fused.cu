@@ -131,7 +131,7 @@ static int fused_setup(const rich_problem_t* pb, int S, FParams& P, int ckpt_eve
         P.ckpt_every = ckpt_every;
         P.keep_states = keep_states;
         P.o_ckpt = off; off = al256(off + (keep_states ? 0 : nc8 * std::max(nck, 1)));
-        P.o_seg = off; off = al256(off + nc8 * (keep_states ? std::max(pb->nsteps, 1) : ckpt_every));
+        P.o_seg = off; off = al256(off + (keep_states ? 0 : nc8 * ckpt_every));
         long long* adj[] = {&P.o_lam, &P.o_rhs, &P.o_r, &P.o_dE, &P.o_dW, &P.o_dN, &P.o_dS, &P.o_dg, &P.o_g,
                             &P.o_rh, &P.o_pk, &P.o_v, &P.o_t, &P.o_ph, &P.o_sh};
         for (long long* o : adj) { *o = (long long)off; off = al256(off + nc8); }
@@ -284,10 +284,15 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     return 0;
 }
 
-// Device memory that the adjoint may use to keep the states of every time step
-// of its resident samples (1.5 % of the GPU's; 152 CTAs of a 256^2 grid keep 50
-// steps in it).  Within it nothing is recomputed and ckpt_every does not matter.
-constexpr size_t KEEP_STATES_BYTES = 4ull << 30;
+// a device buffer of at least `bytes` (what it held is lost when it grows)
+static int grow(void** buf, size_t* have, size_t bytes) {
+    if (*have >= bytes) return 0;
+    if (*buf) cudaFree(*buf);
+    *buf = nullptr; *have = 0;
+    if (cudaMalloc(buf, bytes) != cudaSuccess) { cudaGetLastError(); *buf = nullptr; return RICH_ERR_OOM; }
+    *have = bytes;
+    return 0;
+}
 
 // Discrete adjoint of S samples: QoI and dQ/d ln Ks [S][nz][nx] (g_out).
 int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const double* lnKs,
@@ -298,6 +303,8 @@ int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const dou
     if (ckpt_every < 1 || pb->closure != RICH_GARDNER) return RICH_ERR_INVALID;
     size_t smem = 0;
     int grid = 0, cluster = 0;
+    // the states of all steps where the context's limit and the device's memory
+    // allow them, else the checkpointed layout
     for (bool keep : {true, false}) {
         if (int e = fused_setup(pb, S, P, ckpt_every, keep)) return e;
         // (the GMRES option keeps its small system in one CTA)
@@ -313,17 +320,14 @@ int rich_adjoint_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const dou
         RICH_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 512, smem));
         occ = std::max(occ, 1);
         grid = cluster ? S : std::max(1, std::min(S, ctx->sm_count * occ));
-        if (keep && (size_t)grid * pb->nsteps * pb->nx * pb->nz * 8 > KEEP_STATES_BYTES) continue;
-        const size_t need = (size_t)grid * (size_t)P.slot_bytes + 256;
-        if (ctx->fused_bytes >= need) break;
-        if (ctx->fused_scratch) cudaFree(ctx->fused_scratch);
-        ctx->fused_scratch = nullptr; ctx->fused_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->fused_scratch, need);
-        if (e == cudaSuccess) { ctx->fused_bytes = need; break; }
-        cudaGetLastError();
-        ctx->fused_scratch = nullptr;
-        if (!keep) return RICH_ERR_OOM;               // the checkpointed layout needs less
+        const size_t states = keep ? (size_t)grid * std::max(pb->nsteps, 1) * pb->nx * pb->nz * 8 : 0;
+        if (states > ctx->adj_memory) continue;
+        const int e1 = grow(&ctx->fused_scratch, &ctx->fused_bytes, (size_t)grid * (size_t)P.slot_bytes + 256);
+        const int e2 = e1 ? e1 : grow(&ctx->adj_states, &ctx->adj_states_bytes, states);
+        if (e2 == 0) break;
+        if (!keep) return e2;
     }
+    P.states = (double*)ctx->adj_states;
     P.adj_tol = adj_tol; P.adj_maxit = adj_maxit; P.adj_inner = pb->precision == RICH_MIXED ? 2 : 1;
     P.adj_method = adj_method;
     P.mixed_inner = ctx->tune_mixed_inner > 0 ? ctx->tune_mixed_inner : MIXED_INNER_DEFAULT;

@@ -10,19 +10,20 @@ namespace {
 // Discrete adjoint of the converged time-stepped solve (one sample per CTA):
 // forward with a checkpoint of p every ckpt_every steps, then per segment
 // (last first) recompute its states from the checkpoint and step backwards.
-// With keep_states the forward sweep keeps every step's p instead (one segment)
-// and nothing is recomputed: the second forward solve was nearly half of the
-// call (64^2 x 48 samples x 6 steps: 281 -> 147 ms).  Same bits.
+// With keep_states the forward sweep keeps every step's p instead (one segment, in
+// a buffer of its own) and nothing is recomputed: the second forward solve was
+// nearly half of the call (64^2 x 48 samples x 6 steps: 281 -> 147 ms).  Same bits.
 //   J_N^T lam_N = dQ/dp^N,  J_n^T lam_n = diag(C(p^n)/dt) lam_{n+1},
 //   dQ/dm = dQ/dm|explicit - sum_n (dR_n/dm)^T lam_n     (m = ln Ks).
-// one sample's forward and reverse sweep on its group of threads
+// one sample's forward and reverse sweep on its group of threads, in slot k
 template <typename Gr, typename C_t>
-__device__ __forceinline__ void adjoint_sample(C_t& C, const FParams& P, char* slot, int s) {
+__device__ __forceinline__ void adjoint_sample(C_t& C, const FParams& P, int k, int s) {
+    char* slot = P.scratch + (size_t)k * P.slot_bytes;
     const int nc = C.nc, nx = C.nx, tid = C.tid, nt = C.nt;
     const bool keep = P.keep_states != 0;
     const int CK = keep ? max(P.nsteps, 1) : P.ckpt_every;
     double* ckpt = (double*)(slot + P.o_ckpt);      // [nck][nc]
-    double* seg = (double*)(slot + P.o_seg);        // [CK][nc]
+    double* seg = keep ? P.states + (size_t)k * CK * nc : (double*)(slot + P.o_seg);      // [CK][nc]
     double* lam = (double*)(slot + P.o_lam);
     double* rhs = (double*)(slot + P.o_rhs);
     double* r = (double*)(slot + P.o_r);
@@ -139,7 +140,7 @@ k_adjoint(const FParams P) {
         const int s = s_sample;
         __syncthreads();
         if (s >= P.S) break;
-        adjoint_sample<GCta>(C, P, slot, s);
+        adjoint_sample<GCta>(C, P, blockIdx.x, s);
         __syncthreads();
     }
 }
@@ -170,7 +171,7 @@ k_adjoint_cluster(const FParams P) {
         c.sync();
         const int s = s_sample;
         if (s >= P.S) break;
-        adjoint_sample<GClu>(C, P, slot, s);
+        adjoint_sample<GClu>(C, P, blockIdx.x / n, s);
         c.sync();
     }
 }

@@ -91,6 +91,7 @@ struct FParams {
     int mixed_inner;            // FP32 V-cycles per FP64 defect (mixed path)
     int ckpt_every, keep_states, adj_maxit, adj_inner;
     double adj_tol;
+    double* states;             // keep_states: every step's p, [slot][nsteps][cells]
     long long o_ckpt, o_seg, o_lam, o_rhs, o_r, o_dE, o_dW, o_dN, o_dS, o_dg, o_g;
     int adj_method;             // J^T solver: 0 defect correction, 1 BiCGStab, 2 GMRES(ADJ_M)
     long long o_rh, o_pk, o_v, o_t, o_ph, o_sh;   // BiCGStab vectors

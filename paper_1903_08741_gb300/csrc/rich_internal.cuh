@@ -80,7 +80,13 @@ struct rich_ctx {
     int adj_method = 1;                         // adjoint J^T solver: 0 defect correction, 1 BiCGStab
     double adj_tol = 1e-11;                     // J^T solves: relative residual target ...
     int adj_cap = 400;                          // ... and cap on preconditioner applications
+    size_t adj_memory = 4ull << 30;             // most that a call's kept states may take (1.5 % of the GPU's;
+                                                // 152 CTAs of a 256^2 grid keep 50 steps in it)
+    void* adj_states = nullptr;                 // the kept states; more than ADJ_STATES_POOL of them ...
+    size_t adj_states_bytes = 0;                // ... are freed when the call returns
 };
+
+constexpr size_t ADJ_STATES_POOL = 64ull << 20;
 
 void rich_count_launch();
 int rich_prof_begin(rich_ctx* ctx, cudaStream_t st);
