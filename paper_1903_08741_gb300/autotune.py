@@ -6,7 +6,9 @@ per SM: small grids, whose levels give a large CTA too little work between
 barriers),
 512-thread CTAs (two per
 SM) or 1024-thread CTAs (one per SM: the fewest resident scratch slots, so more
-of the hierarchy stays in L2, and the most threads per sample); for the mixed path
+of the hierarchy stays in L2, and the most threads per sample), and, for few
+samples of a large grid, the library's own choice (0), which gives each sample a
+cluster of CTAs that no set shape does; for the mixed path
 also the number of FP32 V-cycles per FP64 defect (1, 2, 3, 4, 6).  Each
 candidate solves a probe batch of the same grid and precision (fresh seeded
 fields, two time steps) timed with CUDA events.  The probe is the production
@@ -14,9 +16,11 @@ batch itself, up to 64 samples per SM: the persistent kernel balances samples
 of unequal cost through its queue, so a probe with only a few samples per CTA
 is set by its slowest samples and misranks the shapes.  The fastest candidate
 is cached in a JSON file keyed by device, grid, precision and batch size
-(rounded up to a power of two) and applied to the context with
-rich_set_tuning.  Choices measured on GB300 ship with the package
-(tune_defaults.json) and are used when the user cache has no entry.  The
+(rounded up to a power of two; few samples apart) and applied to the context with
+rich_set_tuning, where it stays for later solves of any size: a program that
+solves batches of several sizes tunes for each, or sets 0.  Choices measured on
+GB300 ship with the package (tune_defaults.json) and are used when the user cache
+has no entry.  Entries that other kernels were measured for are not used.  The
 choice never changes an FP64 result (block shape) or the FP64 tolerance
 (inner cycles).
 """
@@ -27,6 +31,7 @@ import os
 import time
 
 
+KERNELS = 2            # generation of the kernels whose measurements hold
 SHIPPED = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tune_defaults.json")
 
 
@@ -45,19 +50,31 @@ def _bucket(n):
     return b
 
 
-def _key(problem, nsamples, device_name):
+def _few(problem, nsamples, sms):
+    """Whether the library may give each sample a cluster of CTAs: V-cycles, a
+    grid of at least 64^2 cells, and at least two SMs a sample."""
+    return problem.cycle <= 1 and problem.nx * problem.nz >= 4096 and 2 * nsamples <= sms
+
+
+def _key(problem, nsamples, device_name, sms=0):
     prec = "mixed" if problem.precision else "fp64"
     cyc = "" if problem.cycle <= 1 else f"|W{problem.cycle}"    # V-cycle keys stay as they were
     clo = "" if problem.closure == 0 else "|VG"
-    return f"{device_name}|{problem.nx}x{problem.nz}|{prec}|S{_bucket(nsamples)}{cyc}{clo}"
+    few = "|few" if _few(problem, nsamples, sms) else ""       # (a bucket may lie on both sides)
+    return f"{device_name}|{problem.nx}x{problem.nz}|{prec}|S{_bucket(nsamples)}{cyc}{clo}{few}"
 
 
-def _load(path):
+def _read(path):
     try:
         with open(path) as f:
             return json.load(f)
     except Exception:
         return {}
+
+
+def _load(path):
+    """The file's entries for the present kernels."""
+    return {k: e for k, e in _read(path).items() if e.get("kernels") == KERNELS}
 
 
 def _save(path, data):
@@ -76,11 +93,23 @@ def shapes(problem):
     return ((32,) if small else ()) + (128, 256, 512, 1024)
 
 
+def candidates(problem, nsamples, sms):
+    """The shapes that tune() times: those of shapes(), and for few samples the
+    library's own choice first, which wins ties."""
+    return ((0,) if _few(problem, nsamples, sms) else ()) + shapes(problem)
+
+
+def _device(device):
+    import torch
+    dev = torch.device(f"cuda:{device}")
+    return dev, torch.cuda.get_device_name(dev), torch.cuda.get_device_properties(dev).multi_processor_count
+
+
 def source(problem, nsamples, device=0):
     """Where tune() would take this key's choice from: "cache", "shipped" or
     "measure"."""
-    import torch
-    key = _key(problem, nsamples, torch.cuda.get_device_name(torch.device(f"cuda:{device}")))
+    _, name, sms = _device(device)
+    key = _key(problem, nsamples, name, sms)
     if key in _load(cache_path()):
         return "cache"
     return "shipped" if key in _load(SHIPPED) else "measure"
@@ -92,18 +121,15 @@ def tune(problem, nsamples, device=0, force=False, probe_steps=2, verbose=False,
     user cache nor (with shipped=True) the package's defaults hold the key."""
     import torch
     import paper_1903_08741_gb300 as R
-    dev = torch.device(f"cuda:{device}")
-    name = torch.cuda.get_device_name(dev)
+    dev, name, sms = _device(device)
     path = cache_path()
-    data = _load(path)
-    key = _key(problem, nsamples, name)
+    key = _key(problem, nsamples, name, sms)
     if not force:
-        for src in (data, _load(SHIPPED) if shipped else {}):
+        for src in (_load(path), _load(SHIPPED) if shipped else {}):
             if key in src:
                 bt, mi = src[key]["block_threads"], src[key]["mixed_inner"]
                 R.set_tuning(bt, mi, device)
                 return bt, mi
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
     S = max(1, min(nsamples, 64 * sms))
     if problem.closure == R.VAN_GENUCHTEN:
         # van Genuchten kernels probe on soil fields of a mid-range soil
@@ -117,7 +143,7 @@ def tune(problem, nsamples, device=0, force=False, probe_steps=2, verbose=False,
     inners = [1, 2, 3, 4, 6] if problem.precision else [0]
     timings = {}
     stream = torch.cuda.current_stream(dev)
-    for bt in shapes(problem):
+    for bt in candidates(problem, nsamples, sms):
         for mi in inners:
             R.set_tuning(bt, mi, device)
             solve(min(S, 8))
@@ -131,9 +157,9 @@ def tune(problem, nsamples, device=0, force=False, probe_steps=2, verbose=False,
                 print(f"tune {key}: block {bt} inner {mi}: {timings[f'{bt}/{mi}']:.1f} ms")
     best = min(timings, key=timings.get)
     bt, mi = (int(x) for x in best.split("/"))
-    data = _load(path)
+    data = _read(path)
     data[key] = {"block_threads": bt, "mixed_inner": mi, "probe_ms": timings, "probe_samples": S,
-                 "probe_steps": probe.nsteps, "when": time.strftime("%Y-%m-%dT%H:%M:%S")}
+                 "probe_steps": probe.nsteps, "kernels": KERNELS, "when": time.strftime("%Y-%m-%dT%H:%M:%S")}
     _save(path, data)
     R.set_tuning(bt, mi, device)
     return bt, mi
@@ -147,7 +173,7 @@ def check(problem, nsamples, device=0, steps=None, verbose=False):
     tuner's shortfall (its time / the best time - 1)."""
     import torch
     import paper_1903_08741_gb300 as R
-    dev = torch.device(f"cuda:{device}")
+    dev, _, sms = _device(device)
     chosen = tune(problem, nsamples, device=device)
     pb = R.Problem(**{**problem.__dict__, "nsteps": steps or problem.nsteps})
     if problem.closure == R.VAN_GENUCHTEN:
@@ -161,7 +187,7 @@ def check(problem, nsamples, device=0, steps=None, verbose=False):
     stream = torch.cuda.current_stream(dev)
     ms = {}
     try:
-        for bt in shapes(problem):
+        for bt in candidates(problem, nsamples, sms):
             for mi in inners:
                 R.set_tuning(bt, mi, device)
                 solve(min(nsamples, 8))
