@@ -491,10 +491,16 @@ static int spectrum_on(rich_ctx* ctx, int px, int pz, double h, const rich_field
     RICH_CUDA(cudaMemcpyAsync(hl.data(), c, sizeof(cplx) * npts, cudaMemcpyDeviceToHost, st));
     RICH_CUDA(cudaStreamSynchronize(st));
     double lmin = hl[0].re, lmax = hl[0].re, sum = 0.0, total = 0.0;
+    for (const cplx& v : hl) { lmin = std::min(lmin, v.re); lmax = std::max(lmax, v.re); }
+    // sums in units of 4^eu, about the largest eigenvalue: they do not overflow
+    // before the eigenvalues do
+    int eu = 0;
+    if (std::isfinite(lmax)) frexp(lmax, &eu);
+    eu = std::max(-500, std::min(500, eu / 2));
+    const double unit = ldexp(1.0, -2 * eu);
     std::vector<double> col(px, 0.0);
     for (int g = 0; g < npts; ++g) {
-        const double v = hl[g].re;
-        lmin = std::min(lmin, v); lmax = std::max(lmax, v);
+        const double v = hl[g].re * unit;
         sum += v;
         if (v > 0.0) { col[g & (px - 1)] += v; total += v; }
     }
@@ -512,12 +518,13 @@ static int spectrum_on(rich_ctx* ctx, int px, int pz, double h, const rich_field
     const bool finite = std::isfinite(sum);               // (an infinite variance: the fields are NaN)
     int etot = 0;
     if (finite) frexp(sqrt(total), &etot);
+    etot += eu;
     int* he = (int*)(hb.data() + o_e);
     int* hsh = (int*)(hb.data() + o_sh);
     const int lx = ilog2(px), lzz = ilog2(pz);
     for (int k = 0; k < px; ++k) {
         he[k] = etot - 62;
-        if (finite && col[k] > 0.0) frexp(sqrt(col[k]), &he[k]);
+        if (finite && col[k] > 0.0) { frexp(sqrt(col[k]), &he[k]); he[k] += eu; }
         he[k] = std::max(he[k], etot - 62);               // below: nothing of it is left in a row
     }
     for (int p = 0; p < px; ++p) {
