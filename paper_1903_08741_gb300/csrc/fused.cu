@@ -232,6 +232,16 @@ static int pick_cluster(const rich_ctx* ctx, const rich_problem_t* pb, int S, FP
     return 0;
 }
 
+// a device buffer of at least `bytes` (what it held is lost when it grows)
+static int grow(void** buf, size_t* have, size_t bytes) {
+    if (*have >= bytes) return 0;
+    if (*buf) cudaFree(*buf);
+    *buf = nullptr; *have = 0;
+    if (cudaMalloc(buf, bytes) != cudaSuccess) { cudaGetLastError(); *buf = nullptr; return RICH_ERR_OOM; }
+    *have = bytes;
+    return 0;
+}
+
 // Fused persistent solve of S samples; stats arrays live in ctx->ws, the
 // per-CTA slots and the queue counter in ctx->fused_scratch.
 int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const double* lnKs,
@@ -259,13 +269,11 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
         if (int e = fused_occupancy(P, smem, nt, &occ)) return e;
         grid = std::max(1, std::min(S, ctx->sm_count * occ));
     }
-    const size_t need = (size_t)grid * off + 256;
-    if (ctx->fused_bytes < need) {
-        if (ctx->fused_scratch) cudaFree(ctx->fused_scratch);
-        ctx->fused_scratch = nullptr; ctx->fused_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->fused_scratch, need);
-        if (e != cudaSuccess) { cudaGetLastError(); return RICH_ERR_OOM; }
-        ctx->fused_bytes = need;
+    // a slot for every CTA that the GPU holds at a time, fewer where memory is short:
+    // the samples come from a queue, so fewer CTAs only take longer
+    while (int e = grow(&ctx->fused_scratch, &ctx->fused_bytes, (size_t)grid * off + 256)) {
+        if (cluster || grid <= ctx->sm_count) return e;
+        grid = std::max(ctx->sm_count, grid / 2);
     }
     P.scratch = (char*)ctx->fused_scratch + 256;
     P.queue = (int*)ctx->fused_scratch;
@@ -281,16 +289,6 @@ int rich_solve_fused(rich_ctx* ctx, const rich_problem_t* pb, int S, const doubl
     w.last = S;
     if (status)
         RICH_CUDA(cudaMemcpyAsync(status, w.status, sizeof(int32_t) * S, cudaMemcpyDeviceToDevice, st));
-    return 0;
-}
-
-// a device buffer of at least `bytes` (what it held is lost when it grows)
-static int grow(void** buf, size_t* have, size_t bytes) {
-    if (*have >= bytes) return 0;
-    if (*buf) cudaFree(*buf);
-    *buf = nullptr; *have = 0;
-    if (cudaMalloc(buf, bytes) != cudaSuccess) { cudaGetLastError(); *buf = nullptr; return RICH_ERR_OOM; }
-    *have = bytes;
     return 0;
 }
 
