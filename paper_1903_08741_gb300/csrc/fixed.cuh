@@ -8,9 +8,12 @@
 // about 30 additions and shifts, on pipes 16 to 32 times as wide.
 //
 // Precision: every value of a transform of white Gaussian noise has a known
-// standard deviation, so one scale for all of them wastes no bits.  It is kept
-// at 2^55 (overflow is at 2^61, more than 22 standard deviations away), so a
-// rounding is 2^-56.8 of the value's deviation, where FP64's is about 2^-54.
+// standard deviation, so one scale for all of them wastes no bits.  It starts at
+// 2^55 and, as the shifts are whole bits, is up to 2^55.5 between the passes of a
+// row and 2^56 between those of a column (behind rows of an odd power of two);
+// inside a pass, before its shift, it is up to 2^57 and 2^57.5.  Overflow is at
+// 2^61: 16 and 11 standard deviations (probabilities of 1e-57 and 1e-29 a value).
+// A rounding is 2^-56.8 of the scale, where FP64's is about 2^-54 of the value.
 #pragma once
 #include <stdint.h>
 #include <math.h>
