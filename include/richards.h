@@ -118,7 +118,8 @@ const char* rich_last_error(void);
  * precision and batch): block_threads 32 (thirty-two resident CTAs per SM,
  * one warp per sample, every level in the sample's slot), 128 (eight), 256
  * (four), 512 (two) or 1024 (one), 0 = chosen from the grid and the batch size
- * (few samples of a large grid: a cluster of two to eight CTAs per sample); mixed_inner = FP32 V-cycles per FP64 defect in
+ * (few samples of a large grid: a cluster of two to eight CTAs per sample, which
+ * no set shape gives them); mixed_inner = FP32 V-cycles per FP64 defect in
  * RICH_MIXED solves, 0 = default 2 (1..16).  The computed solution does not
  * depend on block_threads; mixed_inner changes how often the FP64 stopping
  * test is evaluated (the FP64 tolerance holds either way). */

@@ -211,7 +211,9 @@ static int default_threads(long long nc, int S, int sms) {
 //   mixed: 128^2 x 24 116 / 69 (6; 75 from 64^2), 128^2 x 76 100 / 71 (2; 80),
 //          256^2 x 24 247 / 86 (6; 90)
 // An FP64 half-sweep of a 32^2 level is 1024 clocks of one SM's FP64 pipe, about
-// what the barrier costs; FP32 cells are cheaper, so their line lies higher.
+// what the barrier costs; FP32 cells are cheaper, so their line lies higher.  No
+// finest grid between 32^2 and 64^2 (FP64) or 64^2 and 128^2 (mixed) was measured:
+// such a grid takes no cluster.
 constexpr long long CLUSTER_CELLS64 = 4096, CLUSTER_CELLS32 = 16384;
 
 // CTAs of a sample's cluster (0: one CTA per sample), with the plan of shared

@@ -8,14 +8,17 @@
 // stencil, Eq. five_stencil; red-black Gauss-Seidel; 1/4-sum restriction and
 // piecewise-constant prolongation, Eq. transfer; coarse operators by
 // rediscretisation with arithmetic means of face coefficients, Fig.
-// diffUpscale; exact coarsest solve).  All control flow is per CTA and uniform
-// (decisions come from block-wide reductions), so a sample never waits for
+// diffUpscale; exact coarsest solve).  All control flow is per sample and uniform
+// over its threads (decisions come from reductions over the CTA, or over the
+// cluster of CTAs that shares a sample: gmax, gdot), so a sample never waits for
 // another and there is no host round trip inside a solve.
 //
-// Memory: every CTA owns one scratch slot holding its sample's hierarchy; the
-// slots of the resident CTAs are largely L2 (small grids: L1) resident.
-// Scratch arrays are read with plain loads (they are rewritten inside the
-// kernel; __syncthreads orders the accesses).
+// Memory: every CTA, or cluster of them, owns one scratch slot holding its
+// sample's hierarchy; the slots of the resident CTAs are largely L2 (small grids:
+// L1) resident.  Scratch arrays are read with plain loads: they are rewritten
+// inside the kernel, and __syncthreads orders the accesses of one CTA.  What one
+// CTA of a cluster writes another reads only behind the cluster's barrier
+// (GClu::sync, or gmax and gdot, which hold one).
 //
 // Precision and instruction budget.  GB300 issues 2 FP64 FMAs per SM and
 // clock (1/64 of its FP32 rate), so the FP64 V-cycle is written to minimise
@@ -68,8 +71,9 @@ struct FParams {
     long long osm_alt;                      // likewise the finest level's second red half
     int lw;                                 // first level run by warp 0 alone (nlev: none)
     int lx;                                 // a cluster's sample: levels below lx run on all its CTAs
-    long long s64[MAXL][N64];               // levels >= lw: every array in dynamic shared
-    long long smg[MAXL][NMG];               // memory at these byte offsets (-1: not there)
+    long long s64[MAXL][N64];               // levels below the finest of at most 256 cells: every
+    long long smg[MAXL][NMG];               // array of the cycles in dynamic shared memory at these
+                                            // byte offsets (-1: not there)
     long long smem_bytes;                   // dynamic shared memory of a CTA
     long long o_f64, o_dp64, o_p, o_thold, o_Ks, o_a, o_K, o_th;
     long long slot_bytes;
@@ -652,9 +656,10 @@ __device__ void coarse_factor_warp(int nx, int nz, const T* Tx, const T* Tz, con
 }
 
 // s / u given r = 1/u rounded to nearest: the quotient s r corrected by its
-// exact remainder is the correctly rounded s / u (Markstein, IBM J. Res. Dev.
-// 34, 1990; tiny and huge operands, where the remainder may not be exact, and
-// a zero or non-finite pivot take the division)
+// exact remainder is the correctly rounded s / u, but for quotients within about
+// 2^-52 units of a midpoint (after Markstein, IBM J. Res. Dev. 34, 1990; tiny and
+// huge operands, where the remainder may not be exact, and a zero or non-finite
+// pivot take the division)
 __device__ __forceinline__ double div_by(double s, double u, double r) {
     const double q = s * r;
     const int eq = (__double2hiint(q) >> 20 & 0x7FF) - 1023, eu = (__double2hiint(u) >> 20 & 0x7FF) - 1023;
@@ -850,10 +855,12 @@ __device__ __forceinline__ unsigned long long resid_norm(const Lv<T>& L, bool re
 // ((1 + an) |p|), the Eq. sc_van capacity divided by theta_s - theta_r.  In
 // logarithms: an = exp(n log(a|p|)), S = exp(-m log1p(an)), and since
 // m n = n - 1, (an / (1 + an))^m = an^m S = (an / (a|p|)) S: one exp fewer
-// than exp(m (n log(a|p|) - log1p(an))), and no cancellation between the two
-// logarithms in the dry limit.
+// than exp(m (n log(a|p|) - log1p(an))), and in FP64 no cancellation between the
+// two logarithms in the dry limit.
 // The fixed-point evaluation (fixed.cuh) takes every soil of practice; what
-// leaves its ranges takes the FP64 functions.
+// leaves its ranges takes the FP64 functions.  It does subtract the logarithms,
+// whose errors are absolute and below an FP64 rounding of one: 1 - exp is then off
+// by no more than the rounding of the exp.
 __device__ __forceinline__ double vg_sat(double a, double n, double m, double p) {
     const double ap = -a * p;
     rich_fx::VgLog o;
