@@ -210,6 +210,8 @@ static int default_threads(long long nc, int S, int sms) {
 //          110 from 128^2), 128^2 x 76 181 / 118 (2; 121)
 //   mixed: 128^2 x 24 116 / 69 (6; 75 from 64^2), 128^2 x 76 100 / 71 (2; 80),
 //          256^2 x 24 247 / 86 (6; 90)
+// (how many clusters fit at a time depends on which SMs a GPU has in use: 48 samples took
+// two CTAs each and 24 took five on another)
 // An FP64 half-sweep of a 32^2 level is 1024 clocks of one SM's FP64 pipe, about
 // what the barrier costs; FP32 cells are cheaper, so their line lies higher.  No
 // finest grid between 32^2 and 64^2 (FP64) or 64^2 and 128^2 (mixed) was measured:
